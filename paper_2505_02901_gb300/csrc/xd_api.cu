@@ -213,6 +213,7 @@ static void free_basis(xd_basis_s *b) {
     block_layout_free(b);
     spmm_layout_free(b);
     pass_layout_free(b);
+    win_layout_free(b);
     cudaFree(b->d_hi_off);
     cudaFree(b->d_lo_rank);
     cudaFree(b->d_lo_list);
@@ -352,6 +353,7 @@ xd_status xd_basis_create(int N, int nup, const int32_t *bonds, int nb, const xd
     if (s == XD_OK && b->sym) s = sym_build(b);
     if (s == XD_OK && block_layout_wanted(b)) s = block_layout_build(b);
     if (s == XD_OK && spmm_layout_wanted(b)) s = spmm_layout_build(b);
+    if (s == XD_OK && win_layout_wanted(b)) s = win_layout_build(b);
     if (s != XD_OK) {
         free_basis(b);
         return s;
@@ -473,7 +475,8 @@ static xd_status set_J(xd_ham_s *h, const double *J) {
     if (b->sym) XD_TRY(sym_bond_groups(h));
     if (b->blk.ok) XD_TRY(block_ham_tables(h));
     if (b->spmm.ok) XD_TRY(spmm_ham_tables(h));
-    if (b->spmm.ok) XD_TRY(passes_tables(h));
+    if (b->win.ok) XD_TRY(win_ham_tables(h));
+    if (passes_wanted(b)) XD_TRY(passes_tables(h));
     lanczos_forget(h, false);
     batch_forget(h);  // captured batched launches hold per-coupling scalars
     return XD_OK;
@@ -525,6 +528,7 @@ void xd_ham_destroy(xd_ham h) {
     cudaFree(h->d_dpost);
     cudaFree(h->d_sp_dpost);
     cudaFree(h->d_sp_jhalf);
+    win_ham_free(h);
     cudaFree(h->d_x64_tab);
     cudaFree(h->d_x64_x);
     cudaFree(h->d_x64_state);

@@ -7,6 +7,7 @@
 #include <string>
 #include <vector>
 
+#include "xd_window.h"
 #include "xdiag_gpu.h"
 
 namespace xd {
@@ -140,8 +141,39 @@ struct PassLayoutHost {
     uint64_t *d_pitems[4] = {};          // other prefix bits | window popcount << 32 | rank chunk << 40
     int64_t nitems_p[4] = {};
     std::vector<int> cross_low;          // prefix sites of the cross bonds (lowest in the items' key)
-    uint32_t *d_items[2] = {};           // k_main's items of 4 and of 8 same-class prefixes
-    int64_t nitems[2] = {};
+    uint32_t *d_items = nullptr;         // k_main's items of 4 same-class prefixes
+    int64_t nitems = 0;
+};
+
+// The window passes of a large U(1) block (xd_u1_win.cu).
+struct WinPassDev {
+    WinPass p;
+    WinTables T;                         // the words and slot counts (the lists follow with the couplings)
+    uint64_t *d_whi = nullptr, *d_ohi = nullptr, *d_olo = nullptr;
+    uint32_t *d_olo_off = nullptr;
+    WinSeg *d_segs[5] = {};              // tiles of 1, 2, 4, 8, 16 columns
+    WinCta *d_ctas[5] = {};              // their division among the CTAs
+    WinRun *d_runs[5] = {};
+    int nseg[5] = {}, nctas[5] = {}, nbase[5] = {};
+};
+
+struct WinLayoutHost {
+    bool ok = false;
+    bool spmm32 = false;                     // the FP32 product takes the batched layout (spmm_better)
+    std::vector<std::pair<int, int>> pairs;  // distinct bonds
+    std::vector<int> pair_of;                // per bond
+    std::vector<WinPassDev> pass;
+    unsigned char *buf = nullptr;            // the passes' tables
+};
+
+// One pass's lists, coefficients and diagonals for a Hamiltonian, one allocation.
+struct WinPassHam {
+    unsigned char *buf = nullptr;
+    size_t cap = 0, bytes = 0, oks = 0, osd = 0, ori = 0, oli = 0, ost = 0, ovar = 0;
+    size_t oc[3] = {}, od[3] = {};       // double-float, fixed point, FP32
+    int ng = -1, ncoef = 0, maxslots = 0, maxlist = 0, maxstep = 0;
+    std::vector<int> gid;                // coupling group of every bond of the pass
+    std::vector<uint16_t> slot_word;
 };
 
 }  // namespace xd
@@ -179,6 +211,7 @@ struct xd_basis_s {
     xd::BlockLayoutHost blk;
     xd::SpmmLayoutHost spmm;
     xd::PassLayoutHost pass;
+    xd::WinLayoutHost win;
 
     xd::U1View u1view() const;
     xd::SymView symview() const;
@@ -204,16 +237,20 @@ struct xd_ham_s {
     float *d_sp_dpost = nullptr;    // batched layout: postfix diagonal per class position
     float *d_sp_jhalf = nullptr;    // batched layout: J/2 per bond
     float sp_jcross = 0.f;          // batched layout: sum over cross bonds of J/4
-    // FP64 product on the batched layout without FP64 arithmetic per element
-    // (xd_u1_passes.cu): fixed point when the couplings are small integer
+    // FP64 product on the window passes without FP64 arithmetic per element
+    // (xd_u1_win.cu): fixed point when the couplings are small integer
     // multiples of one quantum, else double-float
+    std::vector<xd::WinPassHam> win;
     bool x64_fx_ok = false;         // the couplings have a quantum: fixed point allowed
+    double x64_qs = 1.0;
+    int x64_B = 0;
+    // small sparse blocks (xd_u1_passes.cu)
     void *d_x64_tab = nullptr;      // one allocation holding the tables below
     void *d_x64_dfc = nullptr, *d_x64_dfd = nullptr, *d_x64_dfp = nullptr;  // double-float: J/2, J/4, postfix diagonal
     void *d_x64_fxc = nullptr, *d_x64_fxd = nullptr, *d_x64_fxp = nullptr;  // fixed point: 2 k_b, k_b, postfix D
     uint32_t *d_x64_post = nullptr; // postfix bond masks | bond << 16
-    double x64_dcross_d = 0.0, x64_qs = 1.0;
-    int x64_dcross_i = 0, x64_B = 0;
+    double x64_dcross_d = 0.0;
+    int x64_dcross_i = 0;
     void *d_x64_x = nullptr;        // workspace, 8 bytes per row (allocated on first use)
     int *d_x64_state = nullptr;     // [E, mode] and the statistics partials
     // first Lanczos pass (xd_lanczos.cu): its stream, device state and, for
@@ -263,13 +300,24 @@ bool spmm_layout_wanted(const xd_basis_s *b);
 xd_status spmm_layout_build(xd_basis_s *b);
 void spmm_layout_free(xd_basis_s *b);
 xd_status spmm_ham_tables(xd_ham_s *h);
-xd_status spmm_apply(const xd_ham_s *h, const void *x, void *y, cudaStream_t st);
-// FP64 product in passes over prefix blocks on the same layout, fixed point
-// or double-float (xd_u1_passes.cu)
+// product in passes over windows of sites (xd_u1_win.cu): FP64 in fixed point
+// or double-float, FP32
+bool win_layout_wanted(const xd_basis_s *b);
+xd_status win_layout_build(xd_basis_s *b);
+void win_layout_free(xd_basis_s *b);
+xd_status win_ham_tables(xd_ham_s *h);
+void win_ham_free(xd_ham_s *h);
+xd_status win_apply_f64(const xd_ham_s *h, const void *x, void *y, cudaStream_t st);
+xd_status win_apply_f32(const xd_ham_s *h, const void *x, void *y, cudaStream_t st);
+// FP64 product of small sparse blocks in passes over prefix blocks (xd_u1_passes.cu)
+bool passes_wanted(const xd_basis_s *b);
 xd_status passes_tables(xd_ham_s *h);
-bool passes_usable(const xd_ham_s *h);
 xd_status passes_apply_f64(const xd_ham_s *h, const void *x, void *y, cudaStream_t st);
 void pass_layout_free(xd_basis_s *b);
+// FP32 product of sparse graphs on the batched layout (xd_u1_spmm.cu)
+bool spmm_better(const xd_basis_s *b);
+xd_status spmm_apply(const xd_ham_s *h, const void *x, void *y, cudaStream_t st);
+xd_status x64_workspace(xd_ham_s *h, int64_t dim);
 // free the FP64 product's workspace (the next FP64 product allocates it again)
 void x64_release(xd_ham_s *h);
 // device allocation for a driver's vectors: when it fails, the handle's FP64

@@ -175,11 +175,11 @@ xd_status u1_states(const xd_basis_s *b, int64_t first, int64_t count, uint64_t 
 
 xd_status u1_apply(const xd_ham_s *h, const void *x, void *y, xd_dtype dt, int nvec,
                    cudaStream_t st) {
-    if (nvec == 1 && dt == XD_F32 && h->b->spmm.ok) return spmm_apply(h, x, y, st);
-    if (nvec == 1 && dt == XD_F64 && passes_usable(h)) {
-        const xd_status s = passes_apply_f64(h, x, y, st);
-        // a workspace that does not fit, or prefix bonds that four windows
-        // cannot hold, send this product to the FP64 block kernel
+    if (nvec == 1 && dt == XD_F32 && h->b->win.spmm32) return spmm_apply(h, x, y, st);
+    if (nvec == 1 && h->b->win.ok) {
+        xd_status s = dt == XD_F64 && passes_wanted(h->b) ? passes_apply_f64(h, x, y, st) : XD_ERANGE;
+        if (s == XD_ERANGE) s = dt == XD_F64 ? win_apply_f64(h, x, y, st) : win_apply_f32(h, x, y, st);
+        // an FP64 workspace or tables (very dense graphs) that do not fit send this product to the block kernel
         if (s != XD_ENOMEM && s != XD_ERANGE) return s;
     }
     if (nvec == 8 && dt == XD_F32 && spmm8_usable(h, x, y)) return spmm8_apply(h, x, y, st);

@@ -363,16 +363,15 @@ void block_layout_free(xd_basis_s *b) {
 xd_status block_ham_tables(xd_ham_s *h) {
     const xd_basis_s *b = h->b;
     const uint32_t nlo = 1u << b->L;
-    std::vector<double> dpost(nlo, 0.0);
-    for (uint32_t g = 0; g < nlo; ++g) {
-        const uint32_t l = b->h_lo_list[g];
-        double d = 0.0;
-        for (int k : b->blk.post) {
-            int i = b->bonds[k].i, j = b->bonds[k].j;
-            d += (((l >> i) & 1) == ((l >> j) & 1) ? 0.25 : -0.25) * h->J[k];
-        }
-        dpost[g] = d;
+    // bond by bond over the words in their natural order, the order in which
+    // each word's terms were always added
+    std::vector<double> by_word(nlo, 0.0), dpost(nlo);
+    for (int k : b->blk.post) {
+        const int i = b->bonds[k].i, j = b->bonds[k].j;
+        const double t[2] = {0.25 * h->J[k], -0.25 * h->J[k]};
+        for (uint32_t l = 0; l < nlo; ++l) by_word[l] += t[((l >> i) ^ (l >> j)) & 1u];
     }
+    for (uint32_t g = 0; g < nlo; ++g) dpost[g] = by_word[b->h_lo_list[g]];
     if (!h->d_dpost) XD_CUDA(dev_malloc((void **)&h->d_dpost, nlo * sizeof(double)));
     XD_CUDA(cudaMemcpy(h->d_dpost, dpost.data(), nlo * sizeof(double), cudaMemcpyHostToDevice));
     return XD_OK;

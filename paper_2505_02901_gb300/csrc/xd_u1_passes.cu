@@ -1,5 +1,9 @@
-// xd_u1_passes.cu -- FP64 y = H x on large U(1) blocks (N >= 24) in passes
-// over prefix blocks, without FP64 arithmetic per matrix element.
+// xd_u1_passes.cu -- FP64 y = H x on small U(1) blocks of sparse graphs
+// (passes_wanted) in passes over prefix blocks, without FP64 arithmetic per
+// matrix element; the window passes of xd_u1_win.cu take over where a row has
+// more flips or the block more rows.  Measured, both sides (us): 24-site chain
+// 122 against 162, 26-site chain with random couplings 529 against 590, 28-site
+// chain 1756 against 1383, 24-site ladder 217 against 183.
 //
 // With the prefix/postfix split of the index layout (Sec. 5.2 two tables,
 // Sec. 5.3 prefix/postfix view) H = H_pre + H_post + H_cross (Eq. 1, pull
@@ -17,35 +21,15 @@
 //     serves KB blocks), items in an order that keeps the cross neighbour
 //     blocks (flips of the prefix sites of cross bonds) in L2.  k_main adds
 //     the passes' sums and the diagonal and writes y.
-// Arithmetic: FP64 input and output (the paper's precision) without FP64
-// arithmetic per element (GB300's FP64 pipe is a small fraction of its FP32
-// and integer rates), in one of two arithmetics chosen per product on the
-// device:
-//     fixed point, for couplings that are small integer multiples k_b q of
-//     one quantum q (e.g. J1 = 1, J2 = 1/2, any uniform model): in units of
-//     q/4 a row is y_r = (q/4) (D(s_r) x_r + sum over flipped b of 2 k_b x_c),
-//     D(s) = sum_b k_b eps_b(s) an integer; x is scaled by 2^S and rounded to
-//     64-bit integers X (|X| < 2^B, no row sum can overflow) and every sum
-//     is exact; each row is converted to FP64 once;
-//     double-float, for any couplings: x is scaled by 2^(1023 - E) (E its
-//     largest biased exponent) and split into FP32 pairs (hi, lo), hi the
-//     top 24 significant bits (exact), lo the next bits rounded to FP32; each
-//     coefficient c is a pair (C, gamma); per element c x is p + e exactly
-//     (p = fl32(C hi), e = fma(C, hi, -p)) plus the small terms C lo + gamma
-//     hi, p enters the accumulator by TwoSum (Knuth) and every rounding error
-//     joins the second word; the row's result 2^(E - 1023) (s + c) costs one
-//     FP64 addition: a relative error near 2^-45 of the sum of the
-//     magnitudes of the row's terms.
-//     A statistics pass (largest exponent and a lower bound of |x|) lets the
-//     device take double-float whenever rounding x to the fixed-point grid
-//     could cost more than 2^-44 |x| (vectors dominated by a few entries).
+// Arithmetic: as xd_u1_win.cu (fixed point or double-float, chosen on the
+// device per product).
 
 #include <algorithm>
-#include <numeric>
 #include <vector>
 
 #include "xd_internal.cuh"
 #include "xd_layout.h"
+#include "xd_x64.cuh"
 
 namespace xd {
 
@@ -67,20 +51,6 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_wait_1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
-// ------------------------------------------------------ double-float pieces
-// (s, c) += (C + gamma) (hi + lo): exact product of the leading parts,
-// TwoSum into s, every rounding error and the small terms into c.
-__device__ __forceinline__ void df_fma(float &s, float &c, float2 C, float2 v) {
-    const float p = __fmul_rn(C.x, v.x);
-    const float e = __fmaf_rn(C.x, v.x, -p);
-    const float low = __fmaf_rn(C.y, v.x, __fmaf_rn(C.x, v.y, e));
-    const float t = __fadd_rn(s, p);
-    const float bp = __fsub_rn(t, s);
-    const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(p, bp));
-    s = t;
-    c = __fadd_rn(c, __fadd_rn(err, low));
-}
-
 // a - b and a + b for pairs: TwoSum of the leading parts, the rest into the low part
 __device__ __forceinline__ float2 df_sub(float2 a, float2 b) {
     const float t = __fsub_rn(a.x, b.x);
@@ -88,47 +58,9 @@ __device__ __forceinline__ float2 df_sub(float2 a, float2 b) {
     const float err = __fadd_rn(__fsub_rn(a.x, __fsub_rn(t, bp)), __fsub_rn(-b.x, bp));
     return make_float2(t, __fadd_rn(err, __fsub_rn(a.y, b.y)));
 }
-__device__ __forceinline__ float2 df_add(float2 a, float2 b) {
-    const float t = __fadd_rn(a.x, b.x);
-    const float bp = __fsub_rn(t, a.x);
-    const float err = __fadd_rn(__fsub_rn(a.x, __fsub_rn(t, bp)), __fsub_rn(b.x, bp));
-    return make_float2(t, __fadd_rn(err, __fadd_rn(a.y, b.y)));
-}
-
-// the double 2^(E - 1023) f, built from the bits of f (exact; subnormal f
-// is taken as zero); E must keep the result in the normal double range
-__device__ __forceinline__ double f2d_scaled(float f, int E) {
-    const uint32_t u = __float_as_uint(f);
-    const int fe = (int)((u >> 23) & 0xffu);
-    const uint64_t sign = (uint64_t)(u >> 31) << 63;
-    if (fe == 0) return __longlong_as_double((long long)sign);
-    return __longlong_as_double((long long)(sign | ((uint64_t)(fe - 127 + E) << 52) | ((uint64_t)(u & 0x7fffffu) << 29)));
-}
-
-// 2^(E - 1023) (s + c).  For 300 <= E <= 1700 both words fold the scale into
-// their exponents exactly (every float exponent stays inside the normal
-// double range) and one FP64 addition rounds the sum.  Otherwise (vectors
-// near the ends of the double range) the unscaled sum is multiplied by
-// 2^(E - 1023) in FP64, which rounds correctly into the subnormal range or
-// to infinity.  E = 2047 (x not finite) gives NaN.
-__device__ __forceinline__ double df_result(float s, float c, int E) {
-    if (E >= 300 && E <= 1700) return f2d_scaled(s, E) + f2d_scaled(c, E);
-    if (E == 2047) return __longlong_as_double(0x7ff8000000000000ll);
-    const double v = f2d_scaled(s, 1023) + f2d_scaled(c, 1023);
-    return v * __longlong_as_double((long long)((uint64_t)E << 52));
-}
-
 __device__ __forceinline__ float2 split_double(double d) {
     const float h = __double2float_rn(d);
     return make_float2(h, __double2float_rn(d - (double)h));
-}
-
-// 2^k as a double for any k (two factors when 2^k is outside the normal range)
-__device__ __forceinline__ double pow2d(int k, double v) {
-    if (k >= -1022 && k <= 1023) return v * __longlong_as_double((long long)((uint64_t)(k + 1023) << 52));
-    const int h = k / 2;
-    v *= __longlong_as_double((long long)((uint64_t)(h + 1023) << 52));
-    return v * __longlong_as_double((long long)((uint64_t)(k - h + 1023) << 52));
 }
 
 
@@ -187,7 +119,6 @@ struct PolFX {
     __device__ static void zero(Acc &a) { a.a = 0; }
     __device__ static V zero_v() { return 0; }
     __device__ static void add(Acc &a, C c, V v) { a.a += (long long)c * v; }
-    __device__ static void add_diff(Acc &a, C c, V nv, V xv) { a.a += (long long)c * (nv - xv); }
     __device__ static void merge(Acc &a, Acc b) { a.a += b.a; }
     __device__ static DA bond_diag(const void *bdiag, const void *, int b) { return __ldg((const int *)bdiag + b); }
     template <class P> __device__ static D block_diag(const P &p, DA d) { return d + p.dcross_i; }
@@ -657,166 +588,7 @@ __global__ void __launch_bounds__(kT, 2) k_main(MainParams p, const typename Pol
     }
 }
 
-// 4^d for d <= 0 in FP32 (0 below the normal range)
-__device__ __forceinline__ float pow4f(int d) { return 2 * d >= -126 ? __uint_as_float((uint32_t)(127 + 2 * d) << 23) : 0.f; }
-
-struct ExpSum {
-    int m;    // largest biased exponent seen
-    float s;  // sum over the entries seen of 4^(e - m), e their biased exponents
-};
-
-__device__ __forceinline__ ExpSum es_join(ExpSum a, ExpSum b) {
-    if (a.m == 2047 || b.m == 2047) return ExpSum{2047, 0.f};
-    const int m = max(a.m, b.m);
-    return ExpSum{m, a.s * pow4f(a.m - m) + b.s * pow4f(b.m - m)};
-}
-
-__device__ ExpSum es_block_reduce(ExpSum v) {
-    __shared__ ExpSum red[32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        ExpSum w;
-        w.m = __shfl_xor_sync(0xffffffffu, v.m, o);
-        w.s = __shfl_xor_sync(0xffffffffu, v.s, o);
-        v = es_join(v, w);
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    __syncthreads();
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        v = lane < nw ? red[lane] : ExpSum{0, 0.f};
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            ExpSum w;
-            w.m = __shfl_xor_sync(0xffffffffu, v.m, o);
-            w.s = __shfl_xor_sync(0xffffffffu, v.s, o);
-            v = es_join(v, w);
-        }
-        if (lane == 0) red[0] = v;
-    }
-    __syncthreads();
-    return red[0];
-}
-
-// Per CTA: the largest biased exponent of its entries of x (2047 when one is
-// infinite or NaN) and sum 4^(e - m) over them, which bounds |x|^2 from
-// below within a factor of 4 (zero and subnormal entries count as zero).
-__global__ void k_x64_stats(const unsigned long long *__restrict__ x, int64_t n, ExpSum *__restrict__ part) {
-    ExpSum v{0, 0.f};
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int e = (int)((__ldg(x + i) >> 52) & 0x7ffull);
-        if (e == 0) continue;
-        if (e == 2047) v.m = 2047;
-        if (v.m == 2047) continue;
-        if (e > v.m) {
-            v.s = v.s * pow4f(v.m - e) + 1.f;
-            v.m = e;
-        } else {
-            v.s += pow4f(e - v.m);
-        }
-    }
-    v = es_block_reduce(v);
-    if (threadIdx.x == 0) part[blockIdx.x] = v;
-}
-
-// Every CTA joins the partials into E (largest biased exponent) and S, and
-// takes the same decision: fixed point when allowed (the couplings have a
-// quantum) and when rounding x to the grid 2^-S of the fixed point, at most
-// sqrt(dim) 2^(E - 1023 - B) in norm, stays below 2^-44 |x| with |x|^2 >=
-// 4^(E - 1023) S, i.e. dim / S <= 4^(B - 44); else double-float.  CTA 0
-// records E and the decision for the product kernels; then x is converted
-// (fixed point: X = round(2^S x), S = B - E + 1022, |X| < 2^B; double-float:
-// (hi, lo) of 2^(1023 - E) x, hi the top 24 significant bits, lo the next 29
-// rounded to FP32).  Subnormal doubles become zero in both.
-__global__ void k_x64_convert(const unsigned long long *__restrict__ x, int64_t n, const ExpSum *__restrict__ part,
-                              int npart, int fx_allowed, int B, int *__restrict__ state, void *__restrict__ out) {
-    ExpSum v{0, 0.f};
-    for (int c = threadIdx.x; c < npart; c += blockDim.x) v = es_join(v, part[c]);
-    v = es_block_reduce(v);
-    const int E = v.m;
-    const bool fx = fx_allowed && E != 2047 && E != 0 &&
-                    (double)n <= (double)v.s * ldexp(1.0, 2 * (B - 44));
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        state[0] = E;
-        state[1] = fx ? 1 : 0;
-    }
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned long long b = __ldg(x + i);
-        const int e = (int)((b >> 52) & 0x7ffull);
-        if (fx) {
-            long long w = 0;
-            if (e != 0) {
-                const unsigned long long M = (b & 0xfffffffffffffull) | (1ull << 52);
-                const int sh = e - E + B - 53;  // 2^S x = M 2^sh, sh <= B - 53
-                if (sh >= 0) w = (long long)(M << sh);
-                else if (sh > -64) w = (long long)((M >> (-sh)) + ((M >> (-sh - 1)) & 1ull));
-                if (b >> 63) w = -w;
-            }
-            ((long long *)out)[i] = w;
-        } else {
-            const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u;
-            const int fe = e - E + 127;  // FP32 exponent field of the scaled value
-            float hi = 0.f, lo = 0.f;
-            if (e != 0 && e != 2047 && fe > 0) {
-                hi = __uint_as_float(sign | ((uint32_t)fe << 23) | (uint32_t)((b >> 29) & 0x7fffffull));
-                const uint32_t r = (uint32_t)(b & 0x1fffffffull);  // value r 2^(fe - 127 - 52)
-                if (r != 0 && fe - 52 > 0)
-                    lo = __uint_as_float(sign | __float_as_uint(__uint2float_rn(r) *
-                                                                __uint_as_float((uint32_t)(fe - 52) << 23)));
-            }
-            ((float2 *)out)[i] = make_float2(hi, lo);
-        }
-    }
-}
-
-
 }  // namespace
-
-// Couplings as small integer multiples of one quantum: J_b = k_b q.  With
-// J_b = m_b 2^e_b (m_b odd), q = gcd(m) 2^(min e); accepted when every |k_b|
-// <= 2^16 and sum |k_b| <= 1365 (so that B >= 47).
-static bool find_quantum(const std::vector<double> &J, double *q, std::vector<int> *k) {
-    int64_t g = 0;
-    int emin = 1 << 20;
-    std::vector<std::pair<int64_t, int>> me;
-    for (double v : J) {
-        if (v == 0.0) {
-            me.push_back({0, 0});
-            continue;
-        }
-        int e = 0;
-        const double f = frexp(v, &e);             // v = f 2^e, 0.5 <= |f| < 1
-        int64_t mm = (int64_t)ldexp(f, 53);        // exact: 53-bit integer
-        e -= 53;
-        while ((mm & 1) == 0) {
-            mm /= 2;
-            ++e;
-        }
-        me.push_back({mm, e});
-        g = std::gcd(g, mm < 0 ? -mm : mm);
-        emin = std::min(emin, e);
-    }
-    k->assign(J.size(), 0);
-    if (g == 0) {
-        *q = 1.0;
-        return true;
-    }
-    int64_t kabs = 0;
-    for (size_t b = 0; b < J.size(); ++b) {
-        if (me[b].first == 0) continue;
-        const int sh = me[b].second - emin;
-        const int64_t mq = me[b].first / g;
-        if (sh > 16 || mq > 65536 || mq < -65536) return false;
-        const int64_t kb = mq * ((int64_t)1 << sh);
-        if (kb > 65536 || kb < -65536) return false;
-        (*k)[b] = (int)kb;
-        kabs += kb < 0 ? -kb : kb;
-        if (kabs > 1365) return false;
-    }
-    *q = ldexp((double)g, emin);
-    return true;
-}
 
 xd_status passes_tables(xd_ham_s *h) {
     const xd_basis_s *b = h->b;
@@ -897,9 +669,6 @@ xd_status passes_tables(xd_ham_s *h) {
     return XD_OK;
 }
 
-
-constexpr int kStatThreads = 256;
-constexpr int kStatPerSm = 8;
 
 // Passes of the prefix bonds and the work items of k_main for this basis,
 // built on first use: windows of at most 12 prefix bits (a tile then holds at
@@ -986,14 +755,11 @@ static xd_status pass_layout_build(xd_basis_s *b) {
     std::sort(cl.begin(), cl.end());
     cl.erase(std::unique(cl.begin(), cl.end()), cl.end());
     pl.cross_low = cl;
-    for (int v = 0; v < 2; ++v) {
-        const int KB = v == 0 ? 4 : 8;
-        const std::vector<uint32_t> items = ordered_items(P, nup, L, KB, kEmpty, cl);
-        pl.nitems[v] = (int64_t)items.size() / KB;
-        XD_CUDA(dev_malloc((void **)&pl.d_items[v], std::max<size_t>(1, items.size()) * sizeof(uint32_t)));
-        if (!items.empty())
-            XD_CUDA(cudaMemcpy(pl.d_items[v], items.data(), items.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
-    }
+    const std::vector<uint32_t> items = ordered_items(P, nup, L, 4, kEmpty, cl);
+    pl.nitems = (int64_t)items.size() / 4;
+    XD_CUDA(dev_malloc((void **)&pl.d_items, std::max<size_t>(1, items.size()) * sizeof(uint32_t)));
+    if (!items.empty())
+        XD_CUDA(cudaMemcpy(pl.d_items, items.data(), items.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
     pl.ok = true;
     return XD_OK;
 }
@@ -1008,40 +774,8 @@ void pass_layout_free(xd_basis_s *b) {
         cudaFree(pl.d_wbond[q]);
         cudaFree(pl.d_pitems[q]);
     }
-    for (int v = 0; v < 2; ++v) cudaFree(pl.d_items[v]);
+    cudaFree(pl.d_items);
     pl = PassLayoutHost();
-}
-
-// The FP64 workspace (8 bytes per row, the two state words and the partials
-// of the statistics pass) is allocated on first use.  When it does not fit,
-// the call returns XD_ENOMEM and this product takes the FP64 block kernel;
-// the next product tries again (the drivers that hold several vectors
-// release the workspace when their own vectors do not fit, x64_release).
-static xd_status x64_workspace(xd_ham_s *h, int64_t dim) {
-    grid_for(1, 1, 1);
-    if (!h->d_x64_state) {
-        cudaError_t e = dev_malloc((void **)&h->d_x64_state, 16 + (size_t)g_num_sms * kStatPerSm * sizeof(ExpSum));
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return XD_ENOMEM;
-        }
-    }
-    if (h->d_x64_x) return XD_OK;
-    cudaError_t e = dev_malloc((void **)&h->d_x64_x, (size_t)dim * 8);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        h->d_x64_x = nullptr;
-        return XD_ENOMEM;
-    }
-    return XD_OK;
-}
-
-void x64_release(xd_ham_s *h) {
-    if (h->d_x64_x) {
-        lanczos_forget(h, false);  // captured Lanczos steps read the workspace
-        cudaFree(h->d_x64_x);
-        h->d_x64_x = nullptr;
-    }
 }
 
 // the passes over the prefix blocks, then k_main, for one arithmetic
@@ -1090,8 +824,8 @@ static xd_status launch_passes(const xd_ham_s *h, const typename Pol::V *x, type
     p.lo_off = s.d_lo_off;
     p.lo_list = s.d_lo_list;
     p.lo_rank = s.d_lo_rank;
-    p.items = pl.d_items[KB == 4 ? 0 : 1];
-    p.nitems = pl.nitems[KB == 4 ? 0 : 1];
+    p.items = pl.d_items;
+    p.nitems = pl.nitems;
     p.xtab = s.d_xtab;
     p.pre = s.d_pre;
     p.npre = s.npre;
@@ -1125,10 +859,10 @@ static xd_status launch_passes(const xd_ham_s *h, const typename Pol::V *x, type
     return XD_OK;
 }
 
-// the batched layout has L = 12 for every block it is built for (N >= 24)
-bool passes_usable(const xd_ham_s *h) {
-    const xd_basis_s *b = h->b;
-    return b->spmm.ok && b->spmm.L == kL && h->d_x64_tab != nullptr;
+// Up to 26 sites and 16 flips to a row, on the batched layout of L = 12
+// (figures at the top).
+bool passes_wanted(const xd_basis_s *b) {
+    return b->spmm.ok && b->spmm.L == kL && b->N <= 26 && win_flips(b->N, b->nup, (int)b->win.pairs.size()) <= 16.0;
 }
 
 // Statistics of x, the choice of arithmetic and the conversion on the
@@ -1139,11 +873,7 @@ xd_status passes_apply_f64(const xd_ham_s *h, const void *x, void *y, cudaStream
     const int64_t dim = h->b->dim;
     XD_TRY(pass_layout_build(h->b));
     XD_TRY(x64_workspace(hm, dim));
-    const int g1 = grid_for(dim, kStatThreads, kStatPerSm);
-    ExpSum *part = (ExpSum *)((unsigned char *)h->d_x64_state + 16);
-    k_x64_stats<<<g1, kStatThreads, 0, st>>>((const unsigned long long *)x, dim, part);
-    k_x64_convert<<<g1, kStatThreads, 0, st>>>((const unsigned long long *)x, dim, part, g1, h->x64_fx_ok ? 1 : 0,
-                                               h->x64_B, h->d_x64_state, h->d_x64_x);
+    x64_convert(h, x, dim, st);
     XD_CUDA(cudaGetLastError());
     if (h->x64_fx_ok) XD_TRY((launch_passes<PolFX, 4>(h, (const long long *)h->d_x64_x, (double *)y, st)));
     return launch_passes<PolDF, 4>(h, (const float2 *)h->d_x64_x, (double *)y, st);

@@ -594,6 +594,19 @@ static xd_status launch_spmm(const xd_ham_s *h, const void *x, void *y, cudaStre
     return XD_OK;
 }
 
+// Sparse graphs, whose products the window passes' fixed cost outweighs: by
+// the estimates of both (this product: 5000 ps a row and 720 a flip, bonds
+// listed twice counted twice).  Measured, this product against the window
+// passes (us): 24-site chain 60 and 100, 26-site chain 194 and 250, 28-site
+// graph of 80 random bonds 2031 and 2450; 28-site chain 699 and 690, 28-site
+// ladder 1596 and 1268, 4x7 lattice 1791 and 1586, 4x8 lattice 31830 and 18130.
+bool spmm_better(const xd_basis_s *b) {
+    if (!b->spmm.ok) return false;
+    std::vector<WinPass> passes;
+    for (const WinPassDev &d : b->win.pass) passes.push_back(d.p);
+    return 5000.0 + 720.0 * win_flips(b->N, b->nup, b->nb) <= win_cost32(b->N, b->nup, passes, (int)b->win.pairs.size());
+}
+
 xd_status spmm_apply(const xd_ham_s *h, const void *x, void *y, cudaStream_t st) {
     switch (h->b->spmm.L) {
         case 10: return launch_spmm<10>(h, x, y, st);
