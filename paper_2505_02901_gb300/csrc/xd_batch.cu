@@ -30,6 +30,7 @@
 
 #include "xd_internal.cuh"
 #include "xd_spmm8.cuh"
+#include "xd_u1_rows.cuh"
 
 namespace xd {
 
@@ -46,18 +47,11 @@ struct Inst {
 
 constexpr int kMaxBatchBonds = 512;
 
-__device__ __forceinline__ uint64_t find_block(const int64_t *__restrict__ hi_off, uint64_t lo,
-                                               uint64_t hi, int64_t r) {
-    while (lo < hi) {
-        uint64_t mid = (lo + hi + 1) >> 1;
-        if (__ldg(hi_off + mid) <= r) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
+using u1rows::find_block;
 
 // Rows [row0, row1) of instance I (bond table staged in sm_mask / sm_half).
-template <typename T, int NV>
-__device__ __forceinline__ void batch_rows(const Inst &I, const uint64_t *sm_mask, const T *sm_half,
+template <typename T, int NV, bool VEC>
+__device__ __forceinline__ void batch_rows_at(const Inst &I, const uint64_t *sm_mask, const T *sm_half,
                                            uint64_t *sh_range, int64_t row0, int64_t row1) {
     const U1View &u = I.u;
     if (threadIdx.x == 0) {
@@ -79,22 +73,25 @@ __device__ __forceinline__ void batch_rows(const Inst &I, const uint64_t *sm_mas
 #pragma unroll
         for (int q = 0; q < NV; ++q) acc[q] = T(0);
         T dsub = T(0);
-        for (int b = 0; b < I.nb; ++b) {
-            const uint64_t mk = sm_mask[b];
-            const uint64_t tt = s & mk;
-            if (tt != 0 && tt != mk) {
-                const uint64_t f = s ^ mk;
-                const int64_t c = __ldg(u.hi_off + (f >> u.L)) + (int64_t)__ldg(u.lo_rank + (f & u.lomask));
-                const T cf = sm_half[b];
-#pragma unroll
-                for (int q = 0; q < NV; ++q) acc[q] += cf * __ldg(x + c * NV + q);
-                dsub += cf;
-            }
-        }
+        // in turn: walked bits spill in k_batch8, whose registers the prefix blocks take
+        u1rows::row_flips<T, NV, false, VEC, false>(u, s, sm_mask, sm_half, I.nb, x, acc, dsub);
         const T d = jq - dsub;
+        T xr[NV];
+        u1rows::load_row<T, NV, false, VEC>(x, r, xr);
 #pragma unroll
-        for (int q = 0; q < NV; ++q) y[r * NV + q] = d * __ldg(x + r * NV + q) + acc[q];
+        for (int q = 0; q < NV; ++q) xr[q] = fma_rn(d, xr[q], acc[q]);
+        u1rows::store_row<T, NV, VEC>(y, r, xr);
     }
+}
+
+// in 16-byte pieces where the instance's vectors allow it
+template <typename T, int NV>
+__device__ __forceinline__ void batch_rows(const Inst &I, const uint64_t *sm_mask, const T *sm_half,
+                                           uint64_t *sh_range, int64_t row0, int64_t row1) {
+    if (u1rows::kVecRow<T, NV> && (((uintptr_t)I.x | (uintptr_t)I.y) & 15) == 0)
+        batch_rows_at<T, NV, u1rows::kVecRow<T, NV>>(I, sm_mask, sm_half, sh_range, row0, row1);
+    else
+        batch_rows_at<T, NV, false>(I, sm_mask, sm_half, sh_range, row0, row1);
 }
 
 // Stages the bond table of instance I.

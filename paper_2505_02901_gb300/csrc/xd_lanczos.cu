@@ -316,15 +316,9 @@ __global__ void __launch_bounds__(kThreads) k_lz_persist(U1View u1, const double
         double d1 = 0.0, d2 = 0.0;
         if (rs.valid) {
             T acc = T(0), dsub = T(0);
-            for (int b = 0; b < nb; ++b) {
-                const uint64_t mk = sm_mask[b];
-                const uint64_t t = rs.s & mk;
-                if (t != 0 && t != mk) {
-                    const T cf = sm_half[b];
-                    acc = fma_rn(cf, __ldcg(u + u1rows::rank_of(u1, rs.s ^ mk)), acc);
-                    dsub += cf;
-                }
-            }
+            T av[1] = {acc};
+            u1rows::row_flips<T, 1, true, false>(u1, rs.s, sm_mask, sm_half, nb, u, av, dsub);
+            acc = av[0];
             const T ur = u[r];
             const T wr = fma_rn(jq - dsub, ur, acc);
             w[r] = wr;

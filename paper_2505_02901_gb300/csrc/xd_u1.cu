@@ -24,7 +24,7 @@ constexpr int kThreads = 256;
 using namespace u1rows;
 
 // y = H x (the row loop of xd_u1_rows.cuh).
-template <typename T, int NV>
+template <typename T, int NV, bool VEC>
 __global__ void __launch_bounds__(kThreads) k_apply(U1View u, const double *__restrict__ bond,
                                                     int nb, const T *__restrict__ x,
                                                     T *__restrict__ y) {
@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(kThreads) k_apply(U1View u, const double *__re
     stage_bonds(bond, nb, sm_mask, sm_half);
     const T jq = (T)bond[2 * nb];
     __syncthreads();
-    apply_rows<T, NV, false>(u, sm_mask, sm_half, nb, jq, x, y, sh_range);
+    apply_rows<T, NV, false, VEC>(u, sm_mask, sm_half, nb, jq, x, y, sh_range);
 }
 
 // State words of rows [first, first + count): the block of row r is the last
@@ -158,7 +158,7 @@ static xd_status launch_apply(const xd_ham_s *h, const void *x, void *y, cudaStr
     const U1View u = h->b->u1view();
     const int nb = h->b->nb;
     size_t smem = (size_t)nb * (sizeof(uint64_t) + sizeof(T));
-    auto kern = k_apply<T, NV>;
+    auto kern = kVecRow<T, NV> && (((uintptr_t)x | (uintptr_t)y) & 15) == 0 ? k_apply<T, NV, kVecRow<T, NV>> : k_apply<T, NV, false>;
     if (smem > 48 * 1024) XD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int grid = grid_for(u.dim, kThreads, 8);
     kern<<<grid, kThreads, smem, st>>>(u, bondbuf, nb, (const T *)x, (T *)y);
