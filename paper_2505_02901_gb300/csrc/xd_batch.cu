@@ -1,5 +1,5 @@
-// xd_batch.cu -- many independent U(1) products in one persistent launch
-// (the multi-vector apply of Sec. 5.1 over a batch of blocks; a9).
+// xd_batch.cu -- many independent U(1) products in one call, the small ones
+// in one persistent launch (the multi-vector apply of Sec. 5.1 over a batch of blocks; a9).
 //
 // Work list: instance k owns ceil(dim_k / tile) row tiles; tile t of the
 // whole batch maps to (instance, first row) through the prefix sums
@@ -15,13 +15,15 @@
 // CUDA graph and replayed while the batch (handles, vectors, dtype, nvec,
 // stream) is unchanged.
 //
-// Eight FP32 right-hand sides with operators large enough for the prefix
-// block layout (N >= 24): one persistent launch of k_batch8 does the whole
-// batch.  Its work list is every prefix block of the large operators (the
-// eight-vector product of xd_u1_spmm8.cu, one block per unit, largest
-// operators first) followed by the row tiles of the small ones; a CTA takes
-// the next unit from a counter in device memory, which the last CTA to
-// finish resets for the next launch.
+// Eight FP32 right-hand sides, operators of N >= 24: one persistent launch of
+// k_batch8 does the small operators and the sparse large ones.  Its work list
+// is every prefix block of the latter (the eight-vector product of
+// xd_u1_spmm8.cu, one block per unit, largest operators first) followed by the
+// row tiles of the small ones; a CTA takes the next unit from a counter in
+// device memory, which the last CTA to finish resets for the next launch.  The
+// other large operators take their window passes (win8_usable, xd_u1_win.cu)
+// one after the other in the same captured graph: they fill the chip by
+// themselves.
 
 #include <algorithm>
 #include <map>
@@ -230,7 +232,8 @@ struct Plan {
     std::vector<const xd_ham_s *> hs;
     std::vector<const void *> xs;
     std::vector<void *> ys;
-    std::vector<int> rest, big;  // small instances (row tiles) / large ones (prefix blocks, k_batch8)
+    std::vector<int> rest, big;  // small instances (row tiles) / large sparse ones (prefix blocks, k_batch8)
+    std::vector<int> win;        // large ones in window passes, one after the other
     xd_dtype dt;
     int nvec;
     cudaStream_t st;
@@ -262,7 +265,8 @@ void launch(const Plan &p, cudaStream_t st) {
     k_batch<T, NV><<<p.grid, p.threads, 0, st>>>(p.d_inst, (int)p.rest.size(), p.ntiles, p.tile_rows);
 }
 
-xd_status launch_any(const Plan &p, cudaStream_t st) {
+// the row tiles and prefix blocks
+xd_status launch_fused(const Plan &p, cudaStream_t st) {
     if (!p.big.empty()) {
         Batch8Args a;
         a.nbig = (int)p.hbig.size();
@@ -290,6 +294,12 @@ xd_status launch_any(const Plan &p, cudaStream_t st) {
         }
     }
     XD_CUDA(cudaGetLastError());
+    return XD_OK;
+}
+
+xd_status launch_any(const Plan &p, cudaStream_t st) {
+    if (!p.big.empty() || !p.rest.empty()) XD_TRY(launch_fused(p, st));
+    for (int k : p.win) XD_TRY(win8_apply(p.hs[k], p.xs[k], p.ys[k], st));
     return XD_OK;
 }
 
@@ -386,10 +396,10 @@ xd_status autotune(Plan *p) {
             p->threads = th;
             p->tile_rows = th * rpt;
             XD_TRY(build_table(p));
-            XD_TRY(launch_any(*p, p->st));  // warm
+            XD_TRY(launch_fused(*p, p->st));  // warm
             XD_CUDA(cudaEventRecord(ev.e[0], p->st));
             for (int r = 0; r < kTuneReps; ++r) {
-                XD_TRY(launch_any(*p, p->st));
+                XD_TRY(launch_fused(*p, p->st));
                 XD_CUDA(cudaEventRecord(ev.e[r + 1], p->st));
             }
             XD_CUDA(cudaEventSynchronize(ev.e[kTuneReps]));
@@ -497,7 +507,9 @@ extern "C" xd_status xd_batch_apply(int ninst, const xd_ham *hs, const void *con
         plan->nvec = nvec;
         plan->st = st;
         for (int k = 0; k < ninst; ++k) {
-            if (dt == XD_F32 && nvec == 8 && (int)plan->big.size() < kMaxBig8 && spmm8_usable(hs[k], xs[k], ys[k]))
+            if (dt == XD_F32 && nvec == 8 && win8_usable(hs[k], xs[k], ys[k]))
+                plan->win.push_back(k);
+            else if (dt == XD_F32 && nvec == 8 && (int)plan->big.size() < kMaxBig8 && spmm8_usable(hs[k], xs[k], ys[k]))
                 plan->big.push_back(k);
             else
                 plan->rest.push_back(k);

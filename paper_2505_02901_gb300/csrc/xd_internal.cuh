@@ -309,6 +309,9 @@ xd_status win_ham_tables(xd_ham_s *h);
 void win_ham_free(xd_ham_s *h);
 xd_status win_apply_f64(const xd_ham_s *h, const void *x, void *y, cudaStream_t st);
 xd_status win_apply_f32(const xd_ham_s *h, const void *x, void *y, cudaStream_t st);
+// eight FP32 right-hand sides, x and y [dim][8], 16-byte aligned
+bool win8_usable(const xd_ham_s *h, const void *x, const void *y);
+xd_status win8_apply(const xd_ham_s *h, const void *x, void *y, cudaStream_t st);
 // FP64 product of small sparse blocks in passes over prefix blocks (xd_u1_passes.cu)
 bool passes_wanted(const xd_basis_s *b);
 xd_status passes_tables(xd_ham_s *h);

@@ -182,6 +182,10 @@ xd_status u1_apply(const xd_ham_s *h, const void *x, void *y, xd_dtype dt, int n
         // an FP64 workspace or tables (very dense graphs) that do not fit send this product to the block kernel
         if (s != XD_ENOMEM && s != XD_ERANGE) return s;
     }
+    if (nvec == 8 && dt == XD_F32 && win8_usable(h, x, y)) {
+        const xd_status s = win8_apply(h, x, y, st);
+        if (s != XD_ERANGE) return s;
+    }
     if (nvec == 8 && dt == XD_F32 && spmm8_usable(h, x, y)) return spmm8_apply(h, x, y, st);
     if (nvec == 1 && h->b->blk.ok) return block_apply(h, x, y, dt, st);
     if (dt == XD_F64) {

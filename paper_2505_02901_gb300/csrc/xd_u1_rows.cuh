@@ -137,35 +137,35 @@ __device__ __forceinline__ void row_flips(const U1View &u, uint64_t s, const uin
                 dsub += cf;
             }
         }
-        return;
-    }
-    for (int b0 = 0; b0 < nb; b0 += 32) {
-        uint32_t fl = 0;
-        const int bn = min(32, nb - b0);
-        for (int b = 0; b < bn; ++b) {
-            const uint64_t mk = sm_mask[b0 + b], t = s & mk;
-            fl |= (uint32_t)(t != 0 && t != mk) << b;
-        }
-        while (fl) {
-            bool on[D];
-            T cf[D], xv[D][NV];
-#pragma unroll
-            for (int d = 0; d < D; ++d) {
-                on[d] = fl != 0;
-                if (on[d]) {
-                    const int b = b0 + __ffs(fl) - 1;
-                    fl &= fl - 1;
-                    cf[d] = sm_half[b];
-                    load_row<T, NV, COHERENT, VEC>(x, rank_of(u, s ^ sm_mask[b]), xv[d]);
-                }
+    } else {
+        for (int b0 = 0; b0 < nb; b0 += 32) {
+            uint32_t fl = 0;
+            const int bn = min(32, nb - b0);
+            for (int b = 0; b < bn; ++b) {
+                const uint64_t mk = sm_mask[b0 + b], t = s & mk;
+                fl |= (uint32_t)(t != 0 && t != mk) << b;
             }
-#pragma unroll
-            for (int d = 0; d < D; ++d)
-                if (on[d]) {
-#pragma unroll
-                    for (int k = 0; k < NV; ++k) acc[k] = fma_rn(cf[d], xv[d][k], acc[k]);
-                    dsub += cf[d];
+            while (fl) {
+                bool on[D];
+                T cf[D], xv[D][NV];
+    #pragma unroll
+                for (int d = 0; d < D; ++d) {
+                    on[d] = fl != 0;
+                    if (on[d]) {
+                        const int b = b0 + __ffs(fl) - 1;
+                        fl &= fl - 1;
+                        cf[d] = sm_half[b];
+                        load_row<T, NV, COHERENT, VEC>(x, rank_of(u, s ^ sm_mask[b]), xv[d]);
+                    }
                 }
+    #pragma unroll
+                for (int d = 0; d < D; ++d)
+                    if (on[d]) {
+    #pragma unroll
+                        for (int k = 0; k < NV; ++k) acc[k] = fma_rn(cf[d], xv[d][k], acc[k]);
+                        dsub += cf[d];
+                    }
+            }
         }
     }
 }

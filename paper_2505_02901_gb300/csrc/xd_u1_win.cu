@@ -168,7 +168,7 @@ struct WinParams {
     const WinK *ks;             // [ws + 1]
     const WinSeg *segs;
     int nseg, c0, co;           // co: columns o of a tile (64 bytes / value size / nv)
-    int nvs, cos;               // log2 of the vectors per row of x and of co
+    int cos;                    // log2 of co
     const WinCta *ctas;
     const WinRun *runs;
     const uint64_t *slot_dep, *whi, *ohi, *olo;
@@ -253,9 +253,11 @@ __device__ __forceinline__ void tile_base(const WinParams &p, const WinTile &T, 
 
 // Rows kind: blocks of RL rows (64 bytes of memory) and CL columns, neighbouring
 // lanes on neighbouring rows.
-template <int VB>
+// WIDE (eight FP32 vectors): blocks of eight rows, a lane's column its 16-byte
+// chunk.
+template <int VB, bool WIDE>
 struct RowBlocks {
-    static constexpr int CW = 64 / VB, CL = VB == 8 ? 4 : 2, RL = 32 / CL, NC = CW / CL;
+    static constexpr int CW = 64 / VB, CL = VB == 8 || WIDE ? 4 : 2, RL = 32 / CL, NC = WIDE ? 1 : CW / CL;
     int nrows, nrb, tot;
     __device__ __forceinline__ RowBlocks(const WinParams &p, const WinTile &T)
         : nrows(__ldg(&p.ks[T.k].nrows)), nrb((nrows + RL - 1) / RL), tot(T.G * nrb) {}
@@ -264,7 +266,7 @@ struct RowBlocks {
         int q = 0;
         while (rb >= (q + 1) * nrb) ++q;
         *g = q;
-        const int r = (rb - q * nrb) * RL + lane % RL;
+        const int r = (rb - q * nrb) * RL + (WIDE ? lane / CL : lane % RL);
         return rb < tot && r < nrows ? rinfo[r] : ~0u;
     }
 };
@@ -390,7 +392,8 @@ __device__ __forceinline__ void row_flips(const unsigned char *tile, const uint2
 
 __device__ __forceinline__ void cp_async_v(void *dst, const void *src, int bytes) {
     const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-    if (bytes == 8) asm volatile("cp.async.ca.shared.global.L2::256B [%0], [%1], 8;\n" ::"r"(d), "l"(src));
+    if (bytes == 16) asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16;\n" ::"r"(d), "l"(src));
+    else if (bytes == 8) asm volatile("cp.async.ca.shared.global.L2::256B [%0], [%1], 8;\n" ::"r"(d), "l"(src));
     else asm volatile("cp.async.ca.shared.global.L2::256B [%0], [%1], 4;\n" ::"r"(d), "l"(src));
 }
 // Hardware barrier `id` of n threads: wait for all, or only be counted.
@@ -403,6 +406,13 @@ __device__ __forceinline__ void bar_arrive(int id, int n) {
     __syncwarp();
     asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(n) : "memory");
 }
+__device__ __forceinline__ void add4(PolF32::Acc (&a)[4], float4 v) {
+    a[0].a += v.x;
+    a[1].a += v.y;
+    a[2].a += v.z;
+    a[3].a += v.w;
+}
+
 template <class T>
 __device__ __forceinline__ T shfl_xor(T v, int mask) {
     union {
@@ -436,19 +446,20 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 // Copies a tile in: the copying warps' part.
-template <class Pol, bool ROWS, typename I>
+template <class Pol, bool ROWS, int NVS, typename I>
 __device__ __forceinline__ void tile_in(const WinParams &p, const WinTile &T, const I *base, const uint8_t *ncol,
                                         unsigned char *tile, const typename Pol::V *x, int ptid) {
     using V = typename Pol::V;
     constexpr int VB = sizeof(V), VL = 16 / VB;
-    const int lane = ptid & 31, nvm = (1 << p.nvs) - 1;
+    constexpr bool WIDE = NVS == 3;
+    const int lane = ptid & 31;
     for (int i = ptid; i < T.G * 8; i += kPT)  // the zero rows
         *(int4 *)(tile + ((i >> 3) * T.nslot + T.nslot - 2) * 64 + (i & 7) * 16) = make_int4(0, 0, 0, 0);
     if constexpr (ROWS) {
-        using R = RowBlocks<VB>;
+        using R = RowBlocks<VB, WIDE>;
         const R rows(p, T);
         const uint32_t *ri = p.rinfo + __ldg(&p.ks[T.k].row0);
-        const int cl = lane / R::RL, nwhi = T.nwhi, unit_bytes = T.nslot * 64;
+        const int cl = WIDE ? lane & 3 : lane / R::RL, nwhi = T.nwhi, unit_bytes = T.nslot * 64;
         constexpr int U = 4;
         for (int rb = ptid >> 5; rb < rows.tot; rb += U * (kPT / 32)) {
             uint32_t e[U];
@@ -464,12 +475,26 @@ __device__ __forceinline__ void tile_in(const WinParams &p, const WinTile &T, co
 #pragma unroll
                 for (int cb = 0; cb < R::NC; ++cb) {
                     const int j = cb * R::CL + cl;
-                    const I b = bw[j >> p.nvs];
+                    const I b = bw[WIDE ? j >> 1 : j];
                     if (b == ~(I)0) continue;
-                    const int64_t q = (((int64_t)b + (e[u] >> 18)) << p.nvs) + (j & nvm);
-                    cp_async_v(row + (ro ^ ((uint32_t)(j & 3) << 4 | (uint32_t)((j >> 2) * VB))), x + q, VB);
+                    const int64_t q = (int64_t)b + (e[u] >> 18);
+                    if constexpr (WIDE) cp_async_v(row + (ro ^ (uint32_t)j << 4), x + 8 * q + 4 * (j & 1), 16);
+                    else cp_async_v(row + (ro ^ ((uint32_t)(j & 3) << 4 | (uint32_t)((j >> 2) * VB))), x + q, VB);
                 }
             }
+        }
+    } else if constexpr (WIDE) {
+        // four lanes to a row of two words o of eight values each
+        const int c = ptid & 3, tot = T.G * kWinRows * T.nstep, cc = T.cc;
+        const bool plain = T.per == 1;
+        const int h = !plain && (c >> 1) >= cc ? 1 : 0, lr = (c >> 1) - h * cc;
+        const float *xl = x + 8 * (int64_t)(T.q0 + lr) + 4 * (c & 1);
+        unsigned char *dst = tile + (ptid >> 2) * 64 + (c << 4);
+        for (int gs = ptid >> 2; gs < tot; gs += kPT / 4, dst += kPT * 16) {
+            const int g = T.lone ? 0 : (int)win_div((uint32_t)gs, T.inv_unit);
+            const int nc = T.lone ? T.nc0 : plain ? (int)ncol[g] : cc;
+            const I b = base[plain ? gs : 2 * gs + h];
+            if (b != ~(I)0 && lr < nc) cp_async_v(dst + g * 128, xl + 8 * (int64_t)b, 16);
         }
     } else {
         // eight lanes to a row, so that a warp access touches four 64-byte
@@ -482,13 +507,13 @@ __device__ __forceinline__ void tile_in(const WinParams &p, const WinTile &T, co
         int lr[NV], h[NV];
 #pragma unroll
         for (int i = 0; i < NV; ++i) {
-            const int jo = (j + 8 * i) >> p.nvs;
+            const int jo = j + 8 * i;
             h[i] = !plain && jo >= cc ? 1 : 0;
             lr[i] = jo - h[i] * cc;
         }
         unsigned char *dst = tile + (ptid >> 3) * 64 + ((j & 3) << 4) + (j >> 2) * VB;
         if (T.lone) {
-            const V *xl = x + ((int64_t)(T.q0 + lr[0]) << p.nvs) + (j & nvm);
+            const V *xl = x + T.q0 + lr[0];
             const bool in0 = lr[0] < T.nc0, in1 = NV > 1 && lr[NV - 1] < T.nc0;
             constexpr int U = 8;
             for (int gs = ptid >> 3; gs < tot; gs += U * (kPT / 8), dst += U * kPT * 8) {
@@ -498,7 +523,7 @@ __device__ __forceinline__ void tile_in(const WinParams &p, const WinTile &T, co
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     if (b[u] == ~(I)0) continue;
-                    const V *src = xl + ((int64_t)b[u] << p.nvs);
+                    const V *src = xl + b[u];
                     if (in0) cp_async_v(dst + u * kPT * 8, src, VB);
                     if (NV > 1 && in1) cp_async_v(dst + u * kPT * 8 + 2 * VB, src + 8, VB);
                 }
@@ -510,7 +535,7 @@ __device__ __forceinline__ void tile_in(const WinParams &p, const WinTile &T, co
                 for (int i = 0; i < NV; ++i) {
                     const I b = base[plain ? gs : 2 * gs + h[i]];
                     if (b != ~(I)0 && lr[i] < nc)
-                        cp_async_v(dst + g * 128 + i * 2 * VB, x + ((((int64_t)b + lr[i]) << p.nvs) + ((j + 8 * i) & nvm)), VB);
+                        cp_async_v(dst + g * 128 + i * 2 * VB, x + ((int64_t)b + lr[i]), VB);
                 }
             }
         }
@@ -529,7 +554,7 @@ __device__ __forceinline__ void tile_in(const WinParams &p, const WinTile &T, co
 // barriers, each tile's buffer with one for "copied" and one for "done with";
 // both roles walk the same tiles, so every wait has its arrivals.  I: uint32
 // row offsets below 2^32 rows.
-template <class Pol, bool ROWS, bool BOND, bool MULTI, typename I>
+template <class Pol, bool ROWS, bool BOND, int NVS, typename I>
 __device__ __forceinline__ void win_pass(const WinParams &p, const typename Pol::V *__restrict__ x,
                                          typename Pol::Acc *acc, typename Pol::Y *y) {
     using V = typename Pol::V;
@@ -537,6 +562,8 @@ __device__ __forceinline__ void win_pass(const WinParams &p, const typename Pol:
     using D = typename Pol::D;
     using Acc = typename Pol::Acc;
     constexpr int VB = sizeof(V), VL = 16 / VB;
+    constexpr bool WIDE = NVS == 3;
+    static_assert(NVS == 0 || (WIDE && VB == 4), "one vector, or eight in FP32");
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ uint8_t ncols[4][64];
     __shared__ WinTile ring[4];  // by tile number
@@ -591,7 +618,7 @@ __device__ __forceinline__ void win_pass(const WinParams &p, const typename Pol:
             }
             bar_sync(kBarCopy, kPT + 32);  // this tile's row offsets and the next one's shape are there
             const WinTile &T = ring[i & 3];
-            tile_in<Pol, ROWS, I>(p, T, base_of(T), ncols[T.gen & 3], smem + (i & 1) * p.sm_tile1, x, ptid);
+            tile_in<Pol, ROWS, NVS, I>(p, T, base_of(T), ncols[T.gen & 3], smem + (i & 1) * p.sm_tile1, x, ptid);
             if (ahead && i + 1 < ntiles) look_up(i + 1);
             cp_async_wait();
             bar_arrive(kBarFull + (i & 1), kMeet);
@@ -602,7 +629,6 @@ __device__ __forceinline__ void win_pass(const WinParams &p, const typename Pol:
     uint2 *steps = (uint2 *)(smem + p.sm_step);
     uint32_t *rinfo = (uint32_t *)(smem + p.sm_rinfo);  // rows kind
     const uint32_t c16 = (uint32_t)(lane & 3) << 4;
-    const int nvm = (1 << p.nvs) - 1;
     const typename Pol::Out oset = Pol::out_setup(p, Pol::kArith < 2 ? __ldg(p.state) : 0);
     int cur = -1, off = 0;  // off: where the deal of steps to warps stands
     const D *diag = nullptr;
@@ -660,7 +686,32 @@ __device__ __forceinline__ void win_pass(const WinParams &p, const typename Pol:
         int o0 = warp - off;
         if (o0 < 0) o0 += kCW;
         off = (off + ntot) % kCW;
-        if constexpr (!ROWS) {
+        if constexpr (!ROWS && WIDE) {
+            const bool plain = T.per == 1, many = plain && !T.lone;
+            const int c = lane & 3, cc = T.cc, cols = plain ? T.nc0 : cc;
+            const int h = !plain && (c >> 1) >= cc ? 1 : 0, lr = (c >> 1) - h * cc;
+            const int64_t shift = 8 * (int64_t)(T.q0 + lr) + 4 * (c & 1);
+            for (int o = o0; o < ntot; o += kCW) {
+                Acc a[2][VL];
+                float4 prev[2];
+                float *at[2];
+                const int nc = many ? (int)ncol[win_div((uint32_t)o, inv_step)] : cols;
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int row = kWinRows * o + (lane >> 2) + 8 * u;
+                    const I b = base[plain ? row : 2 * row + h];
+                    at[u] = b != ~(I)0 && lr < nc ? (float *)y + 8 * (int64_t)b + shift : nullptr;
+                    if (!p.first && at[u]) prev[u] = *(const float4 *)at[u];
+                }
+                step(o, a);
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                    if (at[u]) {
+                        if (!p.first) add4(a[u], prev[u]);
+                        *(float4 *)at[u] = make_float4(a[u][0].a, a[u][1].a, a[u][2].a, a[u][3].a);
+                    }
+            }
+        } else if constexpr (!ROWS) {
             // After its flips a lane trades half of its columns with the lane
             // four on, which has the neighbouring row: then eight lanes hold a
             // row's values and an access touches four 64-byte runs of memory
@@ -675,10 +726,10 @@ __device__ __forceinline__ void win_pass(const WinParams &p, const typename Pol:
                 const int nc = many ? (int)ncol[win_div((uint32_t)o, inv_step)] : cols;
                 // value i of row e of the pair eight u slots on: its index, or false
                 auto place = [&](int u, int e, int i, int64_t *q) -> bool {
-                    const int j = (lane & 3) + 4 * odd + 8 * i, jo = j >> p.nvs, h = !plain && jo >= cc ? 1 : 0;
+                    const int jo = (lane & 3) + 4 * odd + 8 * i, h = !plain && jo >= cc ? 1 : 0;
                     const int lr = jo - (h ? cc : 0), row = gs + 8 * u + e;
                     const I b = base[plain ? row : 2 * row + h];
-                    *q = MULTI ? (((int64_t)b + q0 + lr) << p.nvs) + (j & nvm) : (int64_t)(I)(b + (I)(q0 + lr));
+                    *q = (int64_t)(I)(b + (I)(q0 + lr));
                     return b != ~(I)0 && lr < nc;
                 };
                 if (!p.first)
@@ -741,9 +792,38 @@ __device__ __forceinline__ void win_pass(const WinParams &p, const typename Pol:
             }
             bar_sync(kBarFlip, 32 * kCW);
             // out: the earlier sums of U blocks of rows are read together
-            using R = RowBlocks<VB>;
+            using R = RowBlocks<VB, WIDE>;
             const R rows(p, T);
-            const int cl = lane / R::RL, nwhi = T.nwhi;
+            const int cl = WIDE ? lane & 3 : lane / R::RL, nwhi = T.nwhi;
+            if constexpr (WIDE) {
+                constexpr int U = 4;
+                for (int rb = warp; rb < rows.tot; rb += U * kCW) {
+                    float *at[U];
+                    float4 prev[U];
+                    uint32_t from[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        int g = 0;
+                        const uint32_t e = rb + u * kCW < rows.tot ? rows.row(rinfo, rb + u * kCW, lane, &g) : ~0u;
+                        from[u] = (uint32_t)(g * unit_bytes) + (win_row_off(true, e & 1023u) ^ c16);
+                        const I b = e != ~0u ? base[((g * nwhi + ((e >> 10) & 255u)) << p.cos) + (cl >> 1)] : ~(I)0;
+                        at[u] = b != ~(I)0 ? (float *)y + 8 * ((int64_t)b + (e >> 18)) + 4 * (cl & 1) : nullptr;
+                        if (!p.first && at[u]) prev[u] = *(const float4 *)at[u];
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (at[u]) {
+                            float4 v = *(const float4 *)(tile + from[u]);
+                            if (!p.first) {
+                                v.x += prev[u].x;
+                                v.y += prev[u].y;
+                                v.z += prev[u].z;
+                                v.w += prev[u].w;
+                            }
+                            *(float4 *)at[u] = v;
+                        }
+                }
+            } else {
             constexpr int U = VB == 8 ? 4 : 2;
             for (int rb = warp; rb < rows.tot; rb += U * kCW) {
                 uint32_t row[U];
@@ -758,9 +838,9 @@ __device__ __forceinline__ void win_pass(const WinParams &p, const typename Pol:
 #pragma unroll
                     for (int cb = 0; cb < R::NC; ++cb) {
                         const int j = cb * R::CL + cl;
-                        const I b = e != ~0u ? bw[j >> p.nvs] : ~(I)0;
+                        const I b = e != ~0u ? bw[j] : ~(I)0;
                         idx[u][cb] = b != ~(I)0 ? b + (I)(e >> 18) : b;
-                        if (!p.first && b != ~(I)0) prev[u][cb] = ld_ahead(acc + ((int64_t)idx[u][cb] << p.nvs) + (j & nvm));
+                        if (!p.first && b != ~(I)0) prev[u][cb] = ld_ahead(acc + idx[u][cb]);
                     }
                 }
 #pragma unroll
@@ -769,12 +849,13 @@ __device__ __forceinline__ void win_pass(const WinParams &p, const typename Pol:
                     for (int cb = 0; cb < R::NC; ++cb)
                         if (idx[u][cb] != ~(I)0) {
                             const int j = cb * R::CL + cl;
-                            const int64_t q = ((int64_t)idx[u][cb] << p.nvs) + (j & nvm);
+                            const int64_t q = (int64_t)idx[u][cb];
                             Acc a = *(const Acc *)(tile + (row[u] ^ ((uint32_t)(j & 3) << 4 | (uint32_t)((j >> 2) * VB))));
                             if (!p.first) Pol::merge(a, prev[u][cb]);
                             if (p.last) y[q] = Pol::result(a, oset);
                             else acc[q] = a;
                         }
+            }
             }
         }
         if (i + 2 < ntiles) bar_arrive(kBarEmpty + (i & 1), kMeet);
@@ -782,15 +863,15 @@ __device__ __forceinline__ void win_pass(const WinParams &p, const typename Pol:
 }
 
 // FP64: in the arithmetic that k_x64_convert chose.  FP32: in FP32.
-template <bool F64, bool ROWS, bool BOND, bool MULTI, typename I>
+template <bool F64, bool ROWS, bool BOND, int NVS, typename I>
 __global__ void __launch_bounds__(kT, 1) k_win(const __grid_constant__ WinParams p, const void *__restrict__ x, void *y) {
     if constexpr (F64) {
         if (__ldg(p.state + 1))
-            win_pass<PolFX, ROWS, BOND, MULTI, I>(p, (const long long *)x, (PolFX::Acc *)y, (double *)y);
+            win_pass<PolFX, ROWS, BOND, NVS, I>(p, (const long long *)x, (PolFX::Acc *)y, (double *)y);
         else
-            win_pass<PolDF, ROWS, BOND, MULTI, I>(p, (const float2 *)x, (PolDF::Acc *)y, (double *)y);
+            win_pass<PolDF, ROWS, BOND, NVS, I>(p, (const float2 *)x, (PolDF::Acc *)y, (double *)y);
     } else {
-        win_pass<PolF32, ROWS, BOND, MULTI, I>(p, (const float *)x, (PolF32::Acc *)y, (float *)y);
+        win_pass<PolF32, ROWS, BOND, NVS, I>(p, (const float *)x, (PolF32::Acc *)y, (float *)y);
     }
 }
 
@@ -1040,12 +1121,12 @@ void x64_release(xd_ham_s *h) {
     }
 }
 
-// The passes; nvs = log2 of the vectors per row (MULTI: nvs > 0).
-template <bool F64, bool MULTI>
-static xd_status launch_passes(const xd_ham_s *h, const void *x, void *y, int nvs, cudaStream_t st) {
+// The passes; NVS = log2 of the vectors per row: 0, or 3 in FP32.
+template <bool F64, int NVS>
+static xd_status launch_passes(const xd_ham_s *h, const void *x, void *y, cudaStream_t st) {
     const xd_basis_s *b = h->b;
     const WinLayoutHost &wl = b->win;
-    const int VB = F64 ? 8 : 4, co = (64 / VB) >> nvs;
+    const int VB = F64 ? 8 : 4, co = (64 / VB) >> NVS;
     int cq = 0;
     while ((1 << cq) < co) ++cq;
     const bool wide = b->dim_u1 >= (int64_t)0xffffffffll;
@@ -1064,7 +1145,6 @@ static xd_status launch_passes(const xd_ham_s *h, const void *x, void *y, int nv
         p.runs = d.d_runs[cq];
         p.c0 = d.p.c0;
         p.co = co;
-        p.nvs = nvs;
         p.cos = cq;
         p.slot_dep = (const uint64_t *)(w.buf + w.osd);
         p.ohi = d.d_ohi;
@@ -1112,8 +1192,8 @@ static xd_status launch_passes(const xd_ham_s *h, const void *x, void *y, int nv
         };
         auto pick = [&](auto idx) -> xd_status {
             using I = decltype(idx);
-            if (d.p.rows) return p.ng ? go(k_win<F64, true, false, MULTI, I>) : go(k_win<F64, true, true, MULTI, I>);
-            return p.ng ? go(k_win<F64, false, false, MULTI, I>) : go(k_win<F64, false, true, MULTI, I>);
+            if (d.p.rows) return p.ng ? go(k_win<F64, true, false, NVS, I>) : go(k_win<F64, true, true, NVS, I>);
+            return p.ng ? go(k_win<F64, false, false, NVS, I>) : go(k_win<F64, false, true, NVS, I>);
         };
         XD_TRY(wide ? pick((unsigned long long)0) : pick((unsigned)0));
     }
@@ -1128,11 +1208,29 @@ xd_status win_apply_f64(const xd_ham_s *h, const void *x, void *y, cudaStream_t 
     XD_TRY(x64_workspace(hm, dim));
     x64_convert(h, x, dim, st);
     XD_CUDA(cudaGetLastError());
-    return launch_passes<true, false>(h, h->d_x64_x, y, 0, st);
+    return launch_passes<true, 0>(h, h->d_x64_x, y, st);
 }
 
 xd_status win_apply_f32(const xd_ham_s *h, const void *x, void *y, cudaStream_t st) {
-    return launch_passes<false, false>(h, x, y, 0, st);
+    return launch_passes<false, 0>(h, x, y, st);
+}
+
+// Eight FP32 vectors: where these passes are estimated faster than the prefix
+// blocks of xd_u1_spmm8.cu (ps a row: 26000 a pass and 700 a flip against
+// 28000 and 3600 a flip, bonds listed twice counted twice).  Measured, here
+// and there (us): 28-site ladder 3843 and 6545, 4x7 lattice 5649 and 8507,
+// 24-site ladder 320 and 375; 28-site chain 3527 and 2572, 24-site chain 276
+// and 154.  The dimension keeps every table inside shared memory (32-bit row
+// offsets).
+bool win8_usable(const xd_ham_s *h, const void *x, const void *y) {
+    const xd_basis_s *b = h->b;
+    return b->win.ok && b->dim_u1 < (int64_t)0xffffffffll && (((uintptr_t)x | (uintptr_t)y) & 15) == 0 &&
+           26000.0 * b->win.pass.size() + 700.0 * win_flips(b->N, b->nup, (int)b->win.pairs.size()) <
+               28000.0 + 3600.0 * win_flips(b->N, b->nup, b->nb);
+}
+
+xd_status win8_apply(const xd_ham_s *h, const void *x, void *y, cudaStream_t st) {
+    return launch_passes<false, 3>(h, x, y, st);
 }
 
 }  // namespace xd

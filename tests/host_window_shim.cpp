@@ -30,7 +30,9 @@ int run_pass(const WinPass &p, const WinTables &T, const std::vector<double> &co
     // place of a value in the tile: the unit's bytes, then the row's offset (staging: from the slot; flips: from
     // the list entry) with the column's chunk and place in it
     auto at = [&](int unit_bytes, uint32_t row_off, int j) {
-        const uint32_t o = row_off ^ ((uint32_t)(j & 3) << 4) ^ (uint32_t)((j >> 2) * sh.value_bytes);
+        const bool wide = sh.value_bytes == 4 && sh.nv == 8;  // eight FP32 vectors: four neighbours to a chunk
+        const uint32_t chunk = (uint32_t)(wide ? j >> 2 : j & 3), in = (uint32_t)((wide ? j & 3 : j >> 2) * sh.value_bytes);
+        const uint32_t o = row_off ^ chunk << 4 ^ in;
         return (int64_t)((unit_bytes + o) / sh.value_bytes);
     };
     if (win_div(1023, win_inv(8)) != 127 || win_div(2047, win_inv(255)) != 8) return 19;
