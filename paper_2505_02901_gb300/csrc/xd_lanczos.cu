@@ -93,6 +93,14 @@ struct AccOf<float> {
     using A = AccF;
 };
 
+// Flip tables of the cooperative Lanczos passes: 24 bits of row, 8 of bond,
+// after the bond table in shared memory.
+constexpr int kLzTabRow = 24, kLzTabBonds = 256;
+template <typename T>
+__host__ __device__ inline size_t lz_tab_at(int nb) {
+    return ((size_t)nb * (sizeof(uint64_t) + sizeof(T)) + 15) / 16 * 16;
+}
+
 // Vector updates with their roundings spelt out (a product, then one fused
 // multiply-add), so that every kernel forming a Lanczos vector -- the first
 // pass in any of its forms and the second pass that rebuilds the vectors
@@ -278,35 +286,92 @@ __global__ void __launch_bounds__(kThreads) k_lz_axpby2(int64_t n, T *__restrict
     }
 }
 
+// The product of one row in the cooperative passes below: the row loop's
+// order and roundings (xd_u1_rows.cuh).  TAB: the row's flips are kept in
+// shared memory for the whole pass, target row and bond in one word (column
+// tid of [flips][threads]), so that a step's gathers are independent reads of
+// one vector instead of a chain of table look-ups each.  These passes are
+// bound by the latency of a step: 120 steps of the 16-site ladder 2.27 -> 1.60
+// ms with the table, of the 3x6 lattice (48,620 rows, 72 bonds) 4.05 -> 2.84.
+template <typename T, bool TAB>
+struct LzRow {
+    uint64_t s;
+    bool valid;
+    int n = 0;
+    T dsub = T(0);
+    const uint64_t *mask;
+    const T *half;
+    uint32_t *tab;
+    int nb;
+
+    __device__ __forceinline__ LzRow(const U1View &u1, const double *bond, int nb_, unsigned char *smem, int64_t r,
+                                     uint64_t *sh_range) : nb(nb_) {
+        uint64_t *m = (uint64_t *)smem;
+        T *hf = (T *)(m + nb);
+        u1rows::stage_bonds(bond, nb, m, hf);
+        mask = m;
+        half = hf;
+        tab = (uint32_t *)(smem + lz_tab_at<T>(nb)) + threadIdx.x;
+        const u1rows::RowState rs = u1rows::unrank_tile(u1, (int64_t)blockIdx.x * blockDim.x, r, sh_range);
+        s = rs.s;
+        valid = rs.valid;
+        if (TAB && valid)
+            for (int b = 0; b < nb; ++b) {
+                const uint64_t t = s & mask[b];
+                if (t == 0 || t == mask[b]) continue;
+                tab[kThreads * n++] = (uint32_t)u1rows::rank_of(u1, s ^ mask[b]) | (uint32_t)b << kLzTabRow;
+                dsub += half[b];
+            }
+    }
+    __device__ __forceinline__ T product(const U1View &u1, const T *u, T ur, T jq) const {
+        T acc[1] = {T(0)}, d = dsub;
+        if (TAB) {
+            constexpr int D = 8;
+            for (int j = 0; j < n; j += D) {
+                uint32_t e[D];
+                T x[D];
+#pragma unroll
+                for (int q = 0; q < D; ++q)
+                    if (j + q < n) {
+                        e[q] = tab[kThreads * (j + q)];
+                        x[q] = __ldcg(u + (e[q] & ((1u << kLzTabRow) - 1)));
+                    }
+#pragma unroll
+                for (int q = 0; q < D; ++q)
+                    if (j + q < n) acc[0] = fma_rn(half[e[q] >> kLzTabRow], x[q], acc[0]);
+            }
+        } else {
+            u1rows::row_flips<T, 1, true, false>(u1, s, mask, half, nb, u, acc, d);
+        }
+        return fma_rn(jq - d, ur, acc[0]);
+    }
+};
+
 // The whole first pass in one cooperative launch, for small U(1) blocks
 // whose product is the plain row loop, one row per thread: the row's state
-// word is unranked once and kept in a register.  A step is two phases
-// separated by grid-wide barriers:
-//   product: w_r = (H u)_r in the row loop's order and roundings
-//     (xd_u1_rows.cuh), so that the vectors are those of the second pass bit
-//     for bit, with the partial dots <H u, u> and <up, u>, so that
-//     alpha_k = sig <sig H u + cz up, u> (the modified form) needs no
-//     further pass;
+// word is unranked once (LzRow).  A step is two phases separated by grid-wide
+// barriers:
+//   product: w_r = (H u)_r in the row loop's order and roundings, so that the
+//     vectors are those of the second pass bit for bit, with the partial dots
+//     <H u, u> and <up, u>, so that alpha_k = sig <sig H u + cz up, u> (the
+//     modified form) needs no further pass;
 //   update: w = sig w + cz up - alpha_k sig u, with the partial norms.
 // Every CTA sums the partials itself in the fixed order of warp_sum_parts,
 // so all CTAs hold the same alpha, beta and stop decision; CTA 0 records
 // them.  A thread updates only its own row, so only the product's gathers
 // read other CTAs' writes (through L2).
-template <typename T>
+template <typename T, bool TAB>
 __global__ void __launch_bounds__(kThreads) k_lz_persist(U1View u1, const double *__restrict__ bond, int nb,
                                                          T *b0, T *b1, T *b2, LzDev *sd, double *pa,
                                                          double *pb, double *pc, double *__restrict__ alpha,
                                                          double *__restrict__ beta) {
     cooperative_groups::grid_group grid = cooperative_groups::this_grid();
     extern __shared__ __align__(16) unsigned char smem[];
-    uint64_t *sm_mask = (uint64_t *)smem;
-    T *sm_half = (T *)(sm_mask + nb);
     __shared__ uint64_t sh_range[2];
     __shared__ double sh_sum[2];
-    u1rows::stage_bonds(bond, nb, sm_mask, sm_half);
     const T jq = (T)bond[2 * nb];
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // this thread's row
-    const u1rows::RowState rs = u1rows::unrank_tile(u1, (int64_t)blockIdx.x * blockDim.x, r, sh_range);
+    const LzRow<T, TAB> row(u1, bond, nb, smem, r, sh_range);
     double sig = sd->sig, cz = sd->cz, amax = sd->amax;
     int k = sd->k;
     const int max_iter = sd->max_iter;
@@ -314,13 +379,9 @@ __global__ void __launch_bounds__(kThreads) k_lz_persist(U1View u1, const double
     T *up = b0, *u = b1, *w = b2;
     for (;;) {
         double d1 = 0.0, d2 = 0.0;
-        if (rs.valid) {
-            T acc = T(0), dsub = T(0);
-            T av[1] = {acc};
-            u1rows::row_flips<T, 1, true, false>(u1, rs.s, sm_mask, sm_half, nb, u, av, dsub);
-            acc = av[0];
+        if (row.valid) {
             const T ur = u[r];
-            const T wr = fma_rn(jq - dsub, ur, acc);
+            const T wr = row.product(u1, u, ur, jq);
             w[r] = wr;
             d1 = (double)wr * (double)ur;
             d2 = (double)up[r] * (double)ur;
@@ -341,7 +402,7 @@ __global__ void __launch_bounds__(kThreads) k_lz_persist(U1View u1, const double
         if (rec) alpha[k] = al;
         amax = fmax(amax, fabs(al));
         double d3 = 0.0;
-        if (rs.valid) {
+        if (row.valid) {
             const T t1 = fma_rn((T)cz, up[r], mul_rn((T)sig, w[r]));
             const T t = fma_rn((T)(-al * sig), u[r], t1);
             w[r] = t;
@@ -370,6 +431,45 @@ __global__ void __launch_bounds__(kThreads) k_lz_persist(U1View u1, const double
         sd->k = k;
         sd->done = 1;
     }
+}
+
+// The second pass (eig0) of the same blocks in one cooperative launch: the
+// recurrence with the recorded alpha and beta in the first pass's roundings,
+// psi_r = sum_k coef_k sig_k u_k(r) in a register.  No dots, so one grid-wide
+// barrier a step; the vectors take turns in two buffers.  abc: alpha, beta,
+// coef, [steps] each.  120 steps of the 16-site ladder 3.1 ms as four launches
+// a step, 0.85 ms here; 4x5 lattice (184,756 rows) 12.7 and 8.3 ms.
+template <typename T, bool TAB>
+__global__ void __launch_bounds__(kThreads) k_lz_persist2(U1View u1, const double *__restrict__ bond, int nb, T *b0, T *b1,
+                                                          double sig, int steps, const double *__restrict__ abc,
+                                                          T *__restrict__ psi) {
+    cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint64_t sh_range[2];
+    const T jq = (T)bond[2 * nb];
+    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const LzRow<T, TAB> row(u1, bond, nb, smem, r, sh_range);
+    T *u = b0, *w = b1;
+    T ur = row.valid ? u[r] : T(0), upr = T(0), acc = T(0);
+    double cz = 0.0;
+    for (int k = 0; k < steps; ++k) {
+        acc += (T)(abc[2 * steps + k] * sig) * ur;
+        if (k == steps - 1) break;
+        if (row.valid) {
+            const T wr = row.product(u1, u, ur, jq);
+            const T t = fma_rn((T)(-abc[k] * sig), ur, fma_rn((T)cz, upr, mul_rn((T)sig, wr)));
+            w[r] = t;
+            upr = ur;
+            ur = t;
+        }
+        grid.sync();
+        cz = -abc[steps + k] * sig;
+        sig = 1.0 / abc[steps + k];
+        T *t = u;
+        u = w;
+        w = t;
+    }
+    if (row.valid) psi[r] = acc;
 }
 
 // out[c] = sum over CTAs of part[cta][c], fixed order
@@ -487,27 +587,44 @@ void lanczos_forget(xd_ham_s *h, bool all) {
 struct LzSmall {
     int grid;
     size_t smem;
+    bool tab;  // the rows' flips in shared memory
 };
 
+// Every CTA must be resident: with the flip tables (up to 128 KB a CTA: 127
+// bonds) or else without them.
 template <typename T>
 static bool lz_small_shape(const xd_ham_s *h, LzSmall *out) {
     const xd_basis_s *b = h->b;
     if (b->sym || b->blk.ok || b->spmm.ok || b->dim > (1 << 22)) return false;
-    int dev = 0, coop = 0, per_sm = 0;
-    const size_t smem = (size_t)b->nb * (sizeof(uint64_t) + sizeof(T));
-    if (smem > 48 * 1024 || cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lz_persist<T>, kThreads, smem) != cudaSuccess ||
-        per_sm < 1) {
+    int dev = 0, coop = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) {
         cudaGetLastError();
         return false;
     }
     grid_for(1, 1, 1);
     const int64_t need = (b->dim + kThreads - 1) / kThreads;
-    if (need > (int64_t)per_sm * g_num_sms) return false;
-    out->grid = (int)need;
-    out->smem = smem;
-    return true;
+    for (int tab = 1; tab >= 0; --tab) {
+        if (tab && b->nb > kLzTabBonds) continue;
+        const size_t smem = lz_tab_at<T>(b->nb) + (tab ? (size_t)b->nb * kThreads * sizeof(uint32_t) : 0);
+        if (smem > (tab ? 128 * 1024 : 48 * 1024)) continue;
+        const void *k1 = tab ? (const void *)k_lz_persist<T, true> : (const void *)k_lz_persist<T, false>;
+        const void *k2 = tab ? (const void *)k_lz_persist2<T, true> : (const void *)k_lz_persist2<T, false>;
+        int per1 = 0, per2 = 0;
+        if (cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+            cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per1, k1, kThreads, smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per2, k2, kThreads, smem) != cudaSuccess) {
+            cudaGetLastError();
+            continue;
+        }
+        if (need > (int64_t)std::min(per1, per2) * g_num_sms) continue;
+        out->grid = (int)need;
+        out->smem = smem;
+        out->tab = tab != 0;
+        return true;
+    }
+    return false;
 }
 
 template <typename T>
@@ -521,7 +638,7 @@ static xd_status lanczos_pass1_graph(xd_ham_s *h, int max_iter, uint64_t seed, x
     lw.grid = grid_for(n, kThreads, 8);
     // small blocks whose product is the plain row loop: one cooperative
     // launch for the whole pass (all its CTAs resident at once)
-    LzSmall lzs{0, 0};
+    LzSmall lzs{0, 0, false};
     const bool persist = lz_small_shape<T>(h, &lzs);
     const int pstride = std::max(lw.grid, lzs.grid);  // three arrays of partials
     XD_TRY(ensure_lanczos_partials(h, 3 * pstride));
@@ -583,8 +700,8 @@ static xd_status lanczos_pass1_graph(xd_ham_s *h, int max_iter, uint64_t seed, x
             double *part3 = h->d_lzpart + 2 * pstride;
             void *args[] = {&u1, (void *)&bond, (void *)&nbh, &p0, &p1, &p2, &d_sd, &part1, &part2, &part3, &d_ab,
                             (void *)&d_abb};
-            e = cudaLaunchCooperativeKernel((const void *)k_lz_persist<T>, dim3(lzs.grid), dim3(kThreads), args,
-                                            lzs.smem, st);
+            e = cudaLaunchCooperativeKernel(lzs.tab ? (const void *)k_lz_persist<T, true> : (const void *)k_lz_persist<T, false>,
+                                            dim3(lzs.grid), dim3(kThreads), args, lzs.smem, st);
             if (e == cudaSuccess) e = cudaMemcpyAsync(h_sd, d_sd, sizeof(LzDev), cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
             if (e != cudaSuccess) {
@@ -714,6 +831,32 @@ static xd_status lanczos_run(xd_ham_s *h, int max_iter, uint64_t seed, xd_dtype 
         }
         double sig = 1.0 / sqrt(nrm2), sig_prev = 0.0, beta_prev = 0.0;
         const int steps = *n_iter;
+        LzSmall lzs{0, 0, false};
+        if (lz_small_shape<T>(h, &lzs)) {
+            // the whole pass in one cooperative launch
+            std::vector<double> abc(3 * (size_t)steps);
+            std::copy(alpha, alpha + steps, abc.begin());
+            std::copy(beta, beta + steps, abc.begin() + steps);
+            std::copy(coef, coef + steps, abc.begin() + 2 * (size_t)steps);
+            double *d_abc = nullptr;
+            cudaError_t e = dev_malloc((void **)&d_abc, abc.size() * sizeof(double));
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(d_abc, abc.data(), abc.size() * sizeof(double), cudaMemcpyHostToDevice, st);
+            if (e == cudaSuccess) {
+                int nbh = b->nb, n_steps = steps;
+                U1View u1 = b->u1view();
+                const double *bond = h->d_bond;
+                T *p0 = u, *p1 = w, *out = psi;
+                void *args[] = {&u1, (void *)&bond, &nbh, &p0, &p1, &sig, &n_steps, &d_abc, &out};
+                e = cudaLaunchCooperativeKernel(
+                    lzs.tab ? (const void *)k_lz_persist2<T, true> : (const void *)k_lz_persist2<T, false>, dim3(lzs.grid),
+                    dim3(kThreads), args, lzs.smem, st);
+            }
+            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            cudaFree(d_abc);
+            if (e != cudaSuccess) rc = cuda_status(e, "Lanczos second pass (cooperative)");
+            break;
+        }
         for (int k = 0; k < steps; ++k) {
             k_axpy<T><<<lw.grid, kThreads, 0, st>>>(n, psi, (T)(coef[k] * sig), u);
             cudaError_t e = cudaGetLastError();

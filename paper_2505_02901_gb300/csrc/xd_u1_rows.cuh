@@ -31,7 +31,22 @@ __device__ __forceinline__ uint64_t find_block(const int64_t *__restrict__ hi_of
     return lo;
 }
 
-// Row r -> (state, block).  The CTA first brackets the blocks of its rows.
+// The same by a warp, 32 entries at a time: a search of 2^P entries costs
+// P / 5 dependent reads and not P.
+__device__ __forceinline__ uint64_t find_block_warp(const int64_t *__restrict__ hi_off, uint64_t lo, uint64_t hi, int64_t r) {
+    const uint64_t lane = threadIdx.x & 31;
+    while (lo < hi) {
+        const uint64_t step = (hi - lo + 32) / 32, at = lo + (lane + 1) * step;
+        const uint32_t below = __ballot_sync(0xffffffffu, at <= hi && __ldg(hi_off + (at <= hi ? at : hi)) <= r);
+        lo += __popc(below) * step;
+        hi = min(hi, lo + step - 1);
+    }
+    return lo;
+}
+
+// Row r -> (state, block).  The CTA first brackets the blocks of its rows, its
+// first two warps an end each (product of the 16-site chain, 51 CTAs: 9.4 ->
+// 8.2 us).
 struct RowState {
     uint64_t s;
     bool valid;
@@ -41,13 +56,10 @@ __device__ __forceinline__ RowState unrank_tile(const U1View &u, int64_t base, i
                                                 uint64_t *sh_range) {
     // sh_range[0..1]: block range of rows [base, base + blockDim.x)
     __syncthreads();
-    if (threadIdx.x == 0) {
-        uint64_t nh = 1ull << u.P;
-        int64_t last = min(base + (int64_t)blockDim.x, u.dim) - 1;
-        uint64_t h0 = find_block(u.hi_off, 0, nh - 1, base);
-        uint64_t h1 = find_block(u.hi_off, h0, nh - 1, last);
-        sh_range[0] = h0;
-        sh_range[1] = h1;
+    if (threadIdx.x < 64) {
+        const int64_t last = min(base + (int64_t)blockDim.x, u.dim) - 1;
+        const uint64_t h = find_block_warp(u.hi_off, 0, (1ull << u.P) - 1, threadIdx.x < 32 ? base : last);
+        if ((threadIdx.x & 31) == 0) sh_range[threadIdx.x >> 5] = h;
     }
     __syncthreads();
     RowState rs;
