@@ -52,102 +52,153 @@ __global__ void k_states_range(U1View u, int64_t first, int64_t count, uint64_t 
     }
 }
 
-// Bonds per launch of the bilinear kernel.
-constexpr int kChunk = 256;
+// Bonds per launch of the bilinear kernel, the most that a warp's share of
+// them touches, rows per tile, CTAs per SM.
+constexpr int kChunk = 64, kShare = 5, kBT = 512, kBPer = 4;
+
+struct BilShared {
+    uint64_t s[kBT], mask[kChunk];
+    double g[kBT];
+    long long p[kBT];  // fixed point, or the bits of the double
+    uint16_t list[kBT / 32][kBT];
+    double acc[kBT / 32][kShare][32];  // F_b - F'_b below, a lane's part
+    double red[kBT / 32];
+    uint32_t top[kBT / 32];
+    uint64_t range[2];
+};
 
 // Per-bond bilinear forms: part[cta][b] = sum over the CTA's rows of
 // g_r (S_i.S_j x)_r (Sec. 3.7 inner, per bond).  With p_r = g_r x_r and
 // P = sum_r p_r,
 //   <g|S_i.S_j|x> = 1/4 sum_r eps_b(s_r) p_r + 1/2 sum_{r: b flips} g_r x_c
-//                 = 1/4 (P - 2 F'_b) + 1/2 F_b,
+//                 = 1/4 P + 1/2 (F_b - F'_b),
 // F'_b = sum over flipping rows of p_r and F_b = sum over them of g_r x_c
 // (eps = +1 for parallel, -1 for antiparallel spins): only the flipping
 // bonds of a row cost arithmetic.  A CTA stages the states, g and p of a
-// tile of kBT rows in shared memory; warp w owns bonds w, w + 32, ... of the
-// chunk and every lane walks a fixed set of the tile's rows, so all sums run
-// in a fixed order (lane partials, a fixed shuffle tree, then the CTA
-// partial of each bond).  MBW = most bonds per warp.
-constexpr int kBT = 1024;
-template <typename T, int MBW, bool ZZ>
-__global__ void __launch_bounds__(kBT) k_bilinear_bp(U1View u, const uint64_t *__restrict__ masks,
-                                                     int nb, int b0, const T *__restrict__ g,
-                                                     const T *__restrict__ x,
-                                                     double *__restrict__ part, int nv) {
+// tile of kBT rows in shared memory; the bonds times the tile's 16 groups of
+// 32 rows are dealt to the 16 warps in equal shares, a warp's share being up to
+// kShare neighbouring bonds, the first and last of them in part.  All sums run in
+// a fixed order (lane partials, a fixed shuffle tree, the warps of a bond, then
+// the CTAs).
+//
+// The FP64 pipe (two lanes a clock and SM, idle lanes included) was the limit
+// of one FP64 addition and one FMA for every row and bond with half of the
+// lanes idle.  So a warp first lists the flipping rows of its bond and then
+// takes 32 of them at a time, and F' is summed in integers: p is scaled by a
+// power of two to 58 bits of the tile's largest |p|, whose sums over a lane's
+// 16 rows are exact; the scaling loses less than an FP64 sum of them does.  A
+// tile with an infinity, a NaN or only tiny p (below 2^-965) adds in FP64.
+// The equal shares, sums kept in shared memory and 32 registers (64 warps on
+// an SM) hide the look-ups; more look-ups in flight per lane cost more in idle
+// lanes than they hide (two: 5.3 ms, four: 6.2 below), and a ring of 64 rows in
+// place of the list 5.4.  28-site ladder, 56 bonds: FP64 8.25 -> 4.53 ms, FP32
+// 11.2 -> 6.7 (the conversions); 4x7 lattice, 112 bonds, FP64 14.6 -> 9.1;
+// diagonal part alone (ZZ), 28 pairs 3.7 -> 1.2.
+template <typename T, bool ZZ>
+__global__ void __launch_bounds__(kBT, kBPer)
+    k_bilinear_bp(U1View u, const uint64_t *__restrict__ masks, int nb, int b0, const T *__restrict__ g,
+                  const T *__restrict__ x, double *__restrict__ part, int nv) {
     // nv > 1: column of row-major [dim][nv] vectors (g, x point at the column)
-    __shared__ uint64_t sh_s[kBT];
-    __shared__ double sh_g[kBT], sh_p[kBT];
-    __shared__ double sh_red[kBT / 32];
-    __shared__ uint64_t sh_range[2];
+    constexpr int kWarps = kBT / 32;
+    extern __shared__ __align__(16) unsigned char smem[];
+    BilShared &sh = *(BilShared *)smem;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t below = (1u << lane) - 1;
     const int nbc = min(kChunk, nb - b0);
-    uint64_t mk[MBW];
-    double F[MBW], Fd[MBW];
-#pragma unroll
-    for (int j = 0; j < MBW; ++j) {
-        const int b = warp + 32 * j;
-        mk[j] = b < nbc ? __ldg(masks + b0 + b) : 0ull;
-        F[j] = 0.0;
-        Fd[j] = 0.0;
-    }
+    const int share = warp * nbc, bf = share / kWarps;  // first group of this warp's share, and its bond
+    uint16_t *const list = sh.list[warp];
+    if (tid < nbc) sh.mask[tid] = __ldg(masks + b0 + tid);
+    for (int j = 0; j < kShare; ++j) sh.acc[warp][j][lane] = 0.0;
     double P = 0.0;
     for (int64_t base = (int64_t)blockIdx.x * kBT; base < u.dim; base += (int64_t)gridDim.x * kBT) {
         const int64_t r = base + tid;
-        const RowState rs = unrank_tile(u, base, r, sh_range);
+        const RowState rs = unrank_tile(u, base, r, sh.range);
         const double gr = rs.valid ? (double)g[r * nv] : 0.0;
         const double pr = rs.valid ? gr * (double)x[r * nv] : 0.0;
         P += pr;
-        sh_s[tid] = rs.s;
-        sh_g[tid] = gr;
-        sh_p[tid] = pr;
+        sh.s[tid] = rs.s;  // 0, a state without flips, beyond the last row
+        sh.g[tid] = gr;
+        const uint32_t wtop = __reduce_max_sync(0xffffffffu, (uint32_t)__double2hiint(fabs(pr)) >> 20);
+        if (lane == 0) sh.top[warp] = wtop;
         __syncthreads();
-        const int nrows = (int)min((int64_t)kBT, u.dim - base);
-#pragma unroll 2
-        for (int rr = lane; rr < nrows; rr += 32) {
-            const uint64_t s = sh_s[rr];
-            const double gq = sh_g[rr], pq = sh_p[rr];
+        int top = 0;  // biased exponent of the largest |p|
 #pragma unroll
-            for (int j = 0; j < MBW; ++j) {
-                const uint64_t tb = s & mk[j];
-                if (tb != 0 && tb != mk[j]) {
-                    if (!ZZ) {
-                        const int64_t c = rank_of(u, s ^ mk[j]);
-                        F[j] = fma(gq, (double)__ldg(x + c * nv), F[j]);
-                    }
-                    Fd[j] += pq;
+        for (int w = 0; w < kWarps; ++w) top = max(top, (int)sh.top[w]);
+        const bool fixed = top >= 58 && top < 2047;
+        sh.p[tid] = fixed ? __double2ll_rn(pr * __hiloint2double((2103 - top) << 20, 0)) : __double_as_longlong(pr);
+        const double unit = fixed ? __hiloint2double((top - 57) << 20, 0) : 0.0;
+        __syncthreads();
+        const int steps = (int)(min((int64_t)kBT, u.dim - base) + 31) / 32;
+        for (int j = 0; j < kShare; ++j) {
+            const int k0 = max(0, share - kWarps * (bf + j)), k1 = min(steps, share + nbc - kWarps * (bf + j));
+            if (k0 >= k1) continue;
+            const uint64_t mk = sh.mask[bf + j];
+            double acc = sh.acc[warp][j][lane], direct = 0.0;
+            long long sum = 0;
+            int n = 0;
+#pragma unroll 4
+            for (int k = k0; k < k1; ++k) {
+                const int rr = 32 * k + lane;
+                const uint64_t t = sh.s[rr] & mk;
+                const bool fl = t != 0 && t != mk;
+                if (fl) sum += sh.p[rr];
+                if (!ZZ) {
+                    const uint32_t set = __ballot_sync(0xffffffffu, fl);
+                    if (fl) list[n + __popc(set & below)] = (uint16_t)rr;
+                    n += __popc(set);
                 }
             }
+            if (fixed) {
+                acc = fma((double)sum, -unit, acc);
+            } else {
+#pragma unroll 1
+                for (int k = k0; k < k1; ++k) {
+                    const int rr = 32 * k + lane;
+                    const uint64_t t = sh.s[rr] & mk;
+                    if (t != 0 && t != mk) direct += __longlong_as_double(sh.p[rr]);
+                }
+                acc -= direct;
+            }
+            if (!ZZ) {
+                __syncwarp();
+                for (int i = lane; i < n; i += 32) {
+                    const int rr = list[i];
+                    acc = fma(sh.g[rr], (double)__ldg(x + rank_of(u, sh.s[rr] ^ mk) * nv), acc);
+                }
+                __syncwarp();
+            }
+            sh.acc[warp][j][lane] = acc;
         }
         // the next tile overwrites the staged rows after unrank_tile's barrier
     }
-#pragma unroll
-    for (int j = 0; j < MBW; ++j)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            F[j] += __shfl_xor_sync(0xffffffffu, F[j], o);
-            Fd[j] += __shfl_xor_sync(0xffffffffu, Fd[j], o);
-        }
-#pragma unroll
+    for (int j = 0; j < kShare; ++j) {
+        double v = sh.acc[warp][j][lane];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) sh.acc[warp][j][0] = v;
+    }
     for (int o = 16; o > 0; o >>= 1) P += __shfl_xor_sync(0xffffffffu, P, o);
-    if (lane == 0) sh_red[warp] = P;
+    if (lane == 0) sh.red[warp] = P;
     __syncthreads();
-    double Pb = 0.0;
-    for (int w = 0; w < kBT / 32; ++w) Pb += sh_red[w];
-    if (lane == 0)
-#pragma unroll
-        for (int j = 0; j < MBW; ++j) {
-            const int b = warp + 32 * j;
-            if (b < nbc) part[(size_t)blockIdx.x * nb + b0 + b] = 0.25 * (Pb - 2.0 * Fd[j]) + (ZZ ? 0.0 : 0.5 * F[j]);
+    if (tid < nbc) {
+        double Pb = 0.0, Fb = 0.0;
+        for (int w = 0; w < kWarps; ++w) {
+            Pb += sh.red[w];
+            const int j = tid - w * nbc / kWarps;
+            if (j >= 0 && kWarps * tid < (w + 1) * nbc) Fb += sh.acc[w][j][0];
         }
+        part[(size_t)blockIdx.x * nb + b0 + tid] = 0.25 * Pb + 0.5 * Fb;
+    }
 }
 
-// out[b] = sum_c part[c][b] in fixed order.
+// out[b] = sum_c part[c][b] in fixed order, a warp to a column.
 __global__ void k_sum_columns(const double *__restrict__ part, int rows, int cols,
                               double *__restrict__ out) {
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x & 31;
     if (b >= cols) return;
     double s = 0.0;
-    for (int c = 0; c < rows; ++c) s += part[(size_t)c * cols + b];
-    out[b] = s;
+    for (int c = lane; c < rows; c += 32) s += part[(size_t)c * cols + b];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) out[b] = s;
 }
 
 }  // namespace
@@ -207,16 +258,9 @@ xd_status u1_apply(const xd_ham_s *h, const void *x, void *y, xd_dtype dt, int n
 template <typename T, bool ZZ = false>
 static xd_status launch_bilinear_bp(const U1View &u, const uint64_t *masks, int nb, int grid, const void *g,
                                     const void *x, double *part, cudaStream_t st, int nv = 1) {
+    XD_CUDA(cudaFuncSetAttribute(k_bilinear_bp<T, ZZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BilShared)));
     for (int b0 = 0; b0 < nb; b0 += kChunk) {
-        const int nbc = std::min(kChunk, nb - b0);
-        const int mbw = (nbc + 31) / 32;
-        auto go = [&](auto kern) {
-            kern<<<grid, kBT, 0, st>>>(u, masks, nb, b0, (const T *)g, (const T *)x, part, nv);
-        };
-        if (mbw <= 1) go(k_bilinear_bp<T, 1, ZZ>);
-        else if (mbw <= 2) go(k_bilinear_bp<T, 2, ZZ>);
-        else if (mbw <= 4) go(k_bilinear_bp<T, 4, ZZ>);
-        else go(k_bilinear_bp<T, 8, ZZ>);
+        k_bilinear_bp<T, ZZ><<<grid, kBT, sizeof(BilShared), st>>>(u, masks, nb, b0, (const T *)g, (const T *)x, part, nv);
         XD_CUDA(cudaGetLastError());
     }
     return XD_OK;
@@ -230,7 +274,7 @@ xd_status u1_bilinear_nvec(const xd_ham_s *h, const void *g, const void *x, xd_d
     const xd_basis_s *b = h->b;
     const int nb = b->nb;
     const U1View u = b->u1view();
-    const int grid = grid_for(u.dim, kBT, 1);
+    const int grid = grid_for(u.dim, kBT, kBPer);
     xd_ham_s *hm = const_cast<xd_ham_s *>(h);
     XD_TRY(ensure_partials(hm, sizeof(double) * (size_t)grid * nb * nv));
     const uint64_t *d_masks = (const uint64_t *)(h->d_bond + nb);
@@ -241,7 +285,7 @@ xd_status u1_bilinear_nvec(const xd_ham_s *h, const void *g, const void *x, xd_d
         if (dt == XD_F64) XD_TRY(launch_bilinear_bp<double>(u, d_masks, nb, grid, gk, xk, pk, st, nv));
         else XD_TRY(launch_bilinear_bp<float>(u, d_masks, nb, grid, gk, xk, pk, st, nv));
     }
-    k_sum_columns<<<(nb + 127) / 128, 128, 0, st>>>(hm->d_part, grid * nv, nb, dJ);
+    k_sum_columns<<<(nb + 3) / 4, 128, 0, st>>>(hm->d_part, grid * nv, nb, dJ);
     XD_CUDA(cudaGetLastError());
     return XD_OK;
 }
@@ -251,14 +295,14 @@ xd_status u1_bilinear(const xd_ham_s *h, const void *g, const void *x, xd_dtype 
     const xd_basis_s *b = h->b;
     const int nb = b->nb;
     const U1View u = b->u1view();
-    const int grid = grid_for(u.dim, kBT, 1);
+    const int grid = grid_for(u.dim, kBT, kBPer);
     xd_ham_s *hm = const_cast<xd_ham_s *>(h);
     XD_TRY(ensure_partials(hm, sizeof(double) * (size_t)grid * nb));
     const uint64_t *d_masks = (const uint64_t *)(h->d_bond + nb);
     double *d_part = hm->d_part;
     if (dt == XD_F64) XD_TRY(launch_bilinear_bp<double>(u, d_masks, nb, grid, g, x, d_part, st));
     else XD_TRY(launch_bilinear_bp<float>(u, d_masks, nb, grid, g, x, d_part, st));
-    k_sum_columns<<<(nb + 127) / 128, 128, 0, st>>>(d_part, grid, nb, dJ);
+    k_sum_columns<<<(nb + 3) / 4, 128, 0, st>>>(d_part, grid, nb, dJ);
     XD_CUDA(cudaGetLastError());
     return XD_OK;
 }
@@ -341,12 +385,12 @@ extern "C" xd_status xd_apply_bilinear_noalloc(xd_ham h, const void *g, const vo
     double *part = nullptr;
     XD_TRY(noalloc_scratch(&part));
     const U1View u = b->u1view();
-    const int grid = std::min(grid_for(u.dim, kBT, 1), kNoAllocCtas);
+    const int grid = std::min(grid_for(u.dim, kBT, kBPer), kNoAllocCtas);
     const uint64_t *masks = (const uint64_t *)(h->d_bond + nb);
     cudaStream_t st = (cudaStream_t)stream;
     if (dt == XD_F64) XD_TRY(launch_bilinear_bp<double>(u, masks, nb, grid, g, x, part, st));
     else XD_TRY(launch_bilinear_bp<float>(u, masks, nb, grid, g, x, part, st));
-    k_sum_columns<<<(nb + 127) / 128, 128, 0, st>>>(part, grid, nb, dJ);
+    k_sum_columns<<<(nb + 3) / 4, 128, 0, st>>>(part, grid, nb, dJ);
     XD_CUDA(cudaGetLastError());
     return XD_OK;
 }
@@ -392,7 +436,7 @@ extern "C" xd_status xd_correlations(xd_basis b, const void *psi, xd_dtype dt, c
     }
     if (b->sym) return sym_correlations(b, psi, dt, pairs, npairs, kind, out);
     const U1View u = b->u1view();
-    const int grid = grid_for(u.dim, kBT, 1);
+    const int grid = grid_for(u.dim, kBT, kBPer);
     uint64_t *d_m = nullptr;
     double *d_part = nullptr, *d_out = nullptr;
     cudaError_t e = dev_malloc((void **)&d_m, sizeof(uint64_t) * npairs);
@@ -409,7 +453,7 @@ extern "C" xd_status xd_correlations(xd_basis b, const void *psi, xd_dtype dt, c
                      : launch_bilinear_bp<float, true>(u, d_m, npairs, grid, psi, psi, d_part, 0);
     }
     if (s == XD_OK) {
-        k_sum_columns<<<(npairs + 127) / 128, 128>>>(d_part, grid, npairs, d_out);
+        k_sum_columns<<<(npairs + 3) / 4, 128>>>(d_part, grid, npairs, d_out);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpy(out, d_out, sizeof(double) * npairs, cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) s = cuda_status(e, "xd_correlations");
