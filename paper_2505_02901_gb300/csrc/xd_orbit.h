@@ -323,4 +323,83 @@ XD_HD TorusOrbit torus_orbit(const TorusGeo &g, int ncos, W wk) {
     });
 }
 
+// Ring rotations T_n (i -> i + n mod N) and reflections R_n (i -> n - i mod
+// N): T_n s = rotr(s, n) and R_n s = rotr(rev(s), N - 1 - n) on N-bit words.
+// The smallest image has the longest run of zeros at its top, so only the
+// rotations that bring a longest cyclic zero run of the word there are
+// evaluated.  P_j marks the starts of the runs of length >= j; P_2j = P_j &
+// rotr(P_j, j), and runs >= L + j start where R (runs >= L) & rotr(P_j, L)
+// has a bit, so the longest length takes a doubling and a descent and not a
+// step for every length.  The longest runs of rev(s) are those of s mirrored:
+// the run of s at q .. q + L - 1 is at the top of rotr(s, (q + L) mod N), its
+// mirror image at the top of rotr(rev(s), (N - q) mod N), so both are formed
+// in one loop.  Against a step for every length and a loop for each orientation:
+// product on the 36-site chain 55.5 -> 45.2 ms; a second filter of the runs by
+// the zeros that follow them costs more than the images it saves (43.2 against
+// 39.2 ms in the kernel of its own).  cand (n, or N + n for R_n): the first element reaching rep in
+// the order rotations, then reflections, by ascending run start in the word
+// and in its reversal.
+struct RingOrbit {
+    uint64_t rep;
+    int cand, cnt;
+};
+
+XD_HD uint64_t ring_rev(uint64_t s, int N) {
+#ifdef __CUDA_ARCH__
+    return __brevll(s) >> (64 - N);
+#else
+    uint64_t r = 0;
+    for (int i = 0; i < N; ++i) r |= ((s >> i) & 1) << (N - 1 - i);
+    return r;
+#endif
+}
+
+// rotr by 0 <= j < N of a word, or (no mask) what an AND with N bits leaves of it
+XD_HD uint64_t ring_turn(uint64_t w, int j, int N) { return (w >> j) | (w << ((N - j) & 63)); }
+
+XD_HD RingOrbit ring_orbit(int N, int dih, uint64_t s) {
+    const uint64_t mask = ~0ull >> (64 - N), z = ~s & mask;
+    if (z == 0 || z == mask) return {s, 0, dih ? 2 * N : N};  // every element fixes the word
+    // a P_j with a bit has N > j: no turn below of a word with bits is by N or more
+    const uint64_t p2 = z & ring_turn(z, 1, N), p4 = p2 & ring_turn(p2, 2, N), p8 = p4 & ring_turn(p4, 4, N);
+    uint64_t r = p4 ? p4 : p2 ? p2 : z;
+    int L = p4 ? 4 : p2 ? 2 : 1;
+    if (p8) {
+        const uint64_t p16 = p8 & ring_turn(p8, 8, N), p32 = p16 & ring_turn(p16, 16, N);
+        r = p32 ? p32 : p16 ? p16 : p8;
+        L = p32 ? 32 : p16 ? 16 : 8;
+        uint64_t t = r & ring_turn(p16, L, N);
+        if (t) r = t, L += 16;
+        t = r & ring_turn(p8, L, N);
+        if (t) r = t, L += 8;
+        t = r & ring_turn(p4, L, N);
+        if (t) r = t, L += 4;
+    }
+    uint64_t t = r & ring_turn(p2, L, N);
+    if (t) r = t, L += 2;
+    t = r & ring_turn(z, L, N);
+    if (t) r = t, L += 1;
+    const uint64_t rv = ring_rev(s, N);
+    uint64_t a = ~0ull, b = ~0ull;  // smallest image over the rotations and over the reflections
+    int qa = 0, qb = 0, ca = 0, cb = 0;
+    do {
+        const int q = orb_ctz(r);
+        r &= r - 1;
+        const int n = q + L < N ? q + L : q + L - N;
+        const uint64_t ia = ring_turn(s, n, N) & mask;
+        ca = ia < a ? 1 : ca + (ia == a);
+        qa = ia < a ? n : qa;
+        a = ia < a ? ia : a;
+        if (dih) {
+            // starts in the reversal descend as q does, a run over the end first
+            const uint64_t ib = ((rv << q) | (rv >> ((N - q) & 63))) & mask;
+            qb = ib < b || (ib == b && q + L <= N) ? q : qb;
+            cb = ib < b ? 1 : cb + (ib == b);
+            b = ib < b ? ib : b;
+        }
+    } while (r);
+    if (dih && b < a) return {b, N + (qb ? qb - 1 : N - 1), cb};
+    return {a, qa, ca + (b == a ? cb : 0)};
+}
+
 }  // namespace xd

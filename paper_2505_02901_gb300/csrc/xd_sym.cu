@@ -163,62 +163,10 @@ __device__ __forceinline__ Orbit orbit_min_cosets(const SymView &v, uint64_t s) 
     return o;
 }
 
-// Ring rotations T_n (i -> i + n mod N) and reflections R_n (i -> n - i mod
-// N): T_n s = rotr(s, n) and R_n s = rotr(rev(s), N - 1 - n) on N-bit words.
-// The smallest image has the longest run of zeros at its top, so only the
-// rotations that bring a longest cyclic zero run of the word there are
-// evaluated: z & rotr(z, 1) & ... & rotr(z, L - 1) marks the starts q of the
-// runs of length >= L (z = zero bits of the word), and the run starting at q
-// reaches the top under rotr(., (q + L) mod N).
-__device__ __forceinline__ uint64_t ring_rotr(uint64_t w, int j, int N, uint64_t mask) {
-    return j == 0 ? w : (((w >> j) | (w << (N - j))) & mask);
-}
-
+// Rings: the search of xd_orbit.h.
 __device__ __forceinline__ Orbit orbit_min_ring(const SymView &v, uint64_t s) {
-    const int N = v.cn;
-    const uint64_t mask = N == 64 ? ~0ull : ((1ull << N) - 1);
-    Orbit o{~0ull, 0, 0};
-    for (int refl = 0; refl <= v.cdih; ++refl) {
-        const uint64_t w = refl ? (__brevll(s) >> (64 - N)) : s;
-        const uint64_t z = ~w & mask;
-        if (z == 0) {  // all ones: every element fixes the word
-            o.rep = w;
-            o.u = __ldg(v.cg);
-            o.cnt = v.G;
-            return o;
-        }
-        uint64_t r = z;
-        int L = 1;
-        while (L < N) {
-            const uint64_t r2 = r & ring_rotr(z, L, N, mask);
-            if (!r2) break;
-            r = r2;
-            ++L;
-        }
-        while (r) {
-            const int q = __ffsll((long long)r) - 1;
-            r &= r - 1;
-            int n = q + L;
-            if (n >= N) n -= N;
-            const uint64_t img = ring_rotr(w, n, N, mask);
-            if (img <= o.rep) {
-                int m = n;
-                if (refl) {
-                    m = N - 1 - n;
-                    if (m < 0) m += N;
-                }
-                const int g = __ldg(v.cg + refl * N + m);
-                if (img < o.rep) {
-                    o.rep = img;
-                    o.u = g;
-                    o.cnt = 1;
-                } else {
-                    ++o.cnt;
-                }
-            }
-        }
-    }
-    return o;
+    const RingOrbit t = ring_orbit(v.cn, v.cdih, s);
+    return Orbit{t.rep, (int)__ldg(v.cg + t.cand), t.cnt};
 }
 
 // Narrowing search of xd_orbit.h (tori with at most 8 rows); rowtab in
@@ -448,12 +396,29 @@ __host__ __device__ inline SymBonds symgrp_view(const uint64_t *base, int nb, in
     return v;
 }
 
-template <bool CPLX, bool COS>
+// The representative search of a product.  A kernel holds one of them, so that
+// its registers are those of this search alone: 48 for rings (36-site chain
+// with reflections, ALU bound: 45.2 -> 39.2 ms), and the three smallest rows
+// fit for complex blocks on tori too (6x6 at momentum (pi/3, 0): 412 -> 388
+// ms, real at (0, 0) 361 -> 340).  More resident CTAs by launch bounds (5, 6
+// or 8 to an SM) gave 39 to 41 ms on the chain and 190 to 212 in place of 173
+// with the cosets of the 6x6 triangular lattice.
+enum SymForm {
+    kAnyGroup,   // byte tables, or a torus outside the forms below
+    kRing,       // ring rotations, with or without reflections
+    kRows,       // translations of a torus with rows of at most 7 sites and at most 8 rows
+    kCosetRows,  // the same times point operations
+    kCosets,     // cosets of another torus
+};
+
+template <bool CPLX, SymForm FORM>
 __global__ void __launch_bounds__(kThreads) k_sym_apply(SymView v, SymBonds sbo, int nb, double jq,
                                                         const double *__restrict__ chi,
                                                         const double *__restrict__ sq,
                                                         const typename Val<CPLX>::T *__restrict__ x,
                                                         typename Val<CPLX>::T *__restrict__ y) {
+    constexpr bool COS = FORM == kCosetRows || FORM == kCosets;
+    constexpr bool rows = FORM == kCosetRows || FORM == kRows;  // incremental top step (row states)
     extern __shared__ __align__(16) unsigned char smem[];
     const int ngrp = sbo.ngrp, nchunk = sbo.nchunk;
     uint64_t *sm_smask = (uint64_t *)smem;                   // [nb] sorted bonds
@@ -482,33 +447,29 @@ __global__ void __launch_bounds__(kThreads) k_sym_apply(SymView v, SymBonds sbo,
     for (int q = threadIdx.x; q < 2 * (v.G + 1); q += blockDim.x) sm_sq[q] = sq[q];
     if constexpr (COS)
         for (int q = threadIdx.x; q < (v.tnp - 1) * nb; q += blockDim.x) sm_pm[q] = v.pm[q];
-    const bool narrow = v.tx && v.ty <= 8;
+    const bool narrow = rows || (FORM == kAnyGroup && v.tx && v.ty <= 8);
     if (narrow) {
         for (int q = threadIdx.x; q < (1 << v.tx); q += blockDim.x) sm_rowtab[q] = v.rowtab[q];
         if (v.cut)
             for (int q = threadIdx.x; q < (1 << (2 * v.tx)); q += blockDim.x) sm_cut[q] = v.cut[q];
         for (int q = threadIdx.x; q < max(1, v.tnp) * nb; q += blockDim.x) sm_krow[q] = v.krow[q];
     }
-    // incremental top step (row states, rows of at most 7 sites): translations
-    // alone, or the coset form
-    const bool rows = narrow && v.tx <= 7 && (COS || v.tnp == 0);
     const TorusGeo tgeo = torus_view(v, sm_rowtab, v.cut ? sm_cut : nullptr);
     __syncthreads();
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < v.dim;
          r += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t s = __ldg(v.reps + r);
-        // translations alone, real blocks: the three smallest rows of s; otherwise
-        // the row state of s (the complex form keeps its registers below 64 so)
-        constexpr bool kTop3 = !COS && !CPLX;
+        // translations alone: the three smallest rows of s; otherwise the row state of s
+        constexpr bool kTop3 = !COS;
         uint64_t PM = 0, PA = 0;
         RowTop3 t3;
-        if (rows && kTop3) torus_top3(tgeo, s, t3);
-        else if (rows) torus_rows(tgeo, s, PM, PA);
+        if constexpr (rows && kTop3) torus_top3(tgeo, s, t3);
+        else if constexpr (rows) torus_rows(tgeo, s, PM, PA);
         if constexpr (COS) {
             for (int k = 1; k < v.tnp; ++k) {
                 const uint64_t w = act(v.act, v.nchunk, __ldg(v.tpp + k), s);
                 sm_ps[(k - 1) * kThreads + threadIdx.x] = w;
-                if (rows) {
+                if constexpr (rows) {
                     uint64_t pm, pa;
                     torus_rows(tgeo, w, pm, pa);
                     sm_st[2 * ((k - 1) * kThreads + threadIdx.x)] = pm;
@@ -540,7 +501,7 @@ __global__ void __launch_bounds__(kThreads) k_sym_apply(SymView v, SymBonds sbo,
                     const uint64_t mk = sm_smask[bs];
                     const int b = sm_perm[bs];  // bond id (point-image and row tables)
                     Orbit o;
-                    if (rows) {
+                    if constexpr (rows) {
                         // p_k of the flipped word and its top step: from the three smallest
                         // rows of s (kTop3), or from the row state of p_k s refreshed in the
                         // two rows of the flip
@@ -569,6 +530,8 @@ __global__ void __launch_bounds__(kThreads) k_sym_apply(SymView v, SymBonds sbo,
                         o = coset_search(v, [&](int k) {
                             return k ? sm_ps[(k - 1) * kThreads + threadIdx.x] ^ sm_pm[(k - 1) * nb + b] : s ^ mk;
                         });
+                    } else if constexpr (FORM == kRing) {
+                        o = orbit_min_ring(v, s ^ mk);
                     } else {
                         o = narrow ? orbit_min_narrow(v, tgeo, s ^ mk) : orbit_min(v, s ^ mk);
                     }
@@ -917,12 +880,18 @@ xd_status sym_apply(const xd_ham_s *h, const void *x, void *y, xd_dtype dt, cuda
     // coset form when the point images of the bond masks fit beside the rest
     const bool cos = v.tx && v.tnp > 1 && v.tnp <= kMaxCos && smem_cos <= (size_t)optin;
     if (cos) smem = smem_cos;
+    const bool rows = v.tx && v.tx <= 7 && v.ty <= 8 && (cos || v.tnp == 0);
+    const auto pick = [&](auto cplx) {
+        constexpr bool CPLX = decltype(cplx)::value;
+        return cos ? rows ? k_sym_apply<CPLX, kCosetRows> : k_sym_apply<CPLX, kCosets>
+               : rows ? k_sym_apply<CPLX, kRows> : !v.tx && v.cn ? k_sym_apply<CPLX, kRing> : k_sym_apply<CPLX, kAnyGroup>;
+    };
     if (dt == XD_C128) {
-        auto kern = cos ? k_sym_apply<true, true> : k_sym_apply<true, false>;
+        auto kern = pick(std::true_type());
         XD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         kern<<<grid, kThreads, smem, st>>>(v, sbo, nb, jq, b->d_chi, w.sq, (const double2 *)x, (double2 *)y);
     } else {
-        auto kern = cos ? k_sym_apply<false, true> : k_sym_apply<false, false>;
+        auto kern = pick(std::false_type());
         XD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         kern<<<grid, kThreads, smem, st>>>(v, sbo, nb, jq, b->d_chi, w.sq, (const double *)x, (double *)y);
     }
