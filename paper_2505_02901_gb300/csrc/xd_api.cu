@@ -461,7 +461,7 @@ static xd_status set_J(xd_ham_s *h, const double *J) {
     }
     h->J.assign(J, J + b->nb);
     XD_CUDA(cudaMemcpy(h->d_J, J, sizeof(double) * b->nb, cudaMemcpyHostToDevice));
-    std::vector<double> buf(2 * b->nb + 1);
+    std::vector<double> buf(3 * b->nb + 2);
     double q = 0.0;
     for (int k = 0; k < b->nb; ++k) {
         buf[k] = J[k];
@@ -470,6 +470,17 @@ static xd_status set_J(xd_ham_s *h, const double *J) {
         q += J[k];
     }
     buf[2 * b->nb] = 0.25 * q;
+    // J/2 in units of 2^-62 of a power of two above sum |J/2| (unit 0: not a normal number)
+    double total = 0.0;
+    for (int k = 0; k < b->nb; ++k) total += fabs(0.5 * J[k]);
+    int ex = 0;
+    frexp(total, &ex);
+    const bool fits = isfinite(total) && ex > -900;
+    buf[2 * b->nb + 1] = fits ? ldexp(1.0, ex - 62) : 0.0;
+    for (int k = 0; k < b->nb; ++k) {
+        const long long f = fits ? llrint(ldexp(0.5 * J[k], 62 - ex)) : 0;
+        memcpy(&buf[2 * b->nb + 2 + k], &f, sizeof f);
+    }
     XD_CUDA(cudaMemcpy(h->d_bond, buf.data(), sizeof(double) * buf.size(), cudaMemcpyHostToDevice));
     if (b->sym && !h->d_symtab) XD_TRY(sym_ham_tables(h));
     if (b->sym) XD_TRY(sym_bond_groups(h));
@@ -491,7 +502,7 @@ xd_status xd_ham_create(xd_basis b, const double *J, xd_ham *out) {
     auto *h = new xd_ham_s();
     h->b = b;
     cudaError_t e = dev_malloc((void **)&h->d_J, sizeof(double) * b->nb);
-    if (e == cudaSuccess) e = dev_malloc((void **)&h->d_bond, sizeof(double) * (2 * b->nb + 1));
+    if (e == cudaSuccess) e = dev_malloc((void **)&h->d_bond, sizeof(double) * (3 * b->nb + 2));
     if (e == cudaSuccess) e = dev_malloc((void **)&h->d_scal, sizeof(double) * 64);
     if (e != cudaSuccess) {
         cudaFree(h->d_J);

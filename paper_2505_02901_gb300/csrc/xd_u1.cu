@@ -32,10 +32,12 @@ __global__ void __launch_bounds__(kThreads) k_apply(U1View u, const double *__re
     uint64_t *sm_mask = (uint64_t *)smem;
     T *sm_half = (T *)(sm_mask + nb);
     __shared__ uint64_t sh_range[2];
-    stage_bonds(bond, nb, sm_mask, sm_half);
+    const bool fixed = kFixRow<T> && nb <= kFixBonds && bond[2 * nb + 1] != 0.0;
+    long long *sm_fix = fixed ? (long long *)(sm_half + nb) : nullptr;
+    stage_bonds(bond, nb, sm_mask, sm_half, sm_fix);
     const T jq = (T)bond[2 * nb];
     __syncthreads();
-    apply_rows<T, NV, false, VEC>(u, sm_mask, sm_half, nb, jq, x, y, sh_range);
+    apply_rows<T, NV, false, VEC>(u, sm_mask, sm_half, nb, jq, x, y, sh_range, sm_fix);
 }
 
 // State words of rows [first, first + count): the block of row r is the last
@@ -208,7 +210,7 @@ static xd_status launch_apply(const xd_ham_s *h, const void *x, void *y, cudaStr
     const double *bondbuf = h->d_bond;
     const U1View u = h->b->u1view();
     const int nb = h->b->nb;
-    size_t smem = (size_t)nb * (sizeof(uint64_t) + sizeof(T));
+    size_t smem = (size_t)nb * (sizeof(uint64_t) + sizeof(T)) + (kFixRow<T> && nb <= kFixBonds ? (nb + 1) * sizeof(long long) : 0);
     auto kern = kVecRow<T, NV> && (((uintptr_t)x | (uintptr_t)y) & 15) == 0 ? k_apply<T, NV, kVecRow<T, NV>> : k_apply<T, NV, false>;
     if (smem > 48 * 1024) XD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int grid = grid_for(u.dim, kThreads, 8);

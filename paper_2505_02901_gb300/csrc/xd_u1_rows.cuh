@@ -124,19 +124,29 @@ __device__ __forceinline__ void store_row(T *y, int64_t r, const T (&v)[NV]) {
 }
 
 // The flipping bonds of a row with state s, in ascending order: acc += J_b/2
-// x_c for each of the NV columns and dsub += J_b/2.  Rows of 32 bytes and more
-// (WALK): the bonds are tested 32 at a time and then only the set bits are
-// walked, two targets being read together, so that a warp runs as long as its
-// row with the most flips and not once for every bond with half of its lanes
-// idle; the FP64 pipe, the limit for eight columns, costs a warp the same
-// whether lanes are idle or not.  4x6 lattice, eight columns: FP64 3058 ->
-// 2612 us; 22-site ladder, FP32 175 -> 105 us.  Narrower rows take every bond
-// in turn: the test is most of their work (22-site ladder, two FP32 columns: 52
-// us in turn, 66 us walked).
-template <typename T, int NV, bool COHERENT, bool VEC, bool WALK = (NV * sizeof(T) >= 32)>
+// x_c for each of the NV columns and dsub += J_b/2.  FP64 rows and rows of 32
+// bytes and more (WALK): the bonds are tested 32 at a time and then only the
+// set bits are walked, two targets being read together, so that a warp runs as
+// long as its row with the most flips and not once for every bond with half of
+// its lanes idle; the FP64 pipe, the limit in FP64, costs a warp the same
+// whether lanes are idle or not.  fix (or null; [nb], and then the unit): J_b/2
+// in integers, so that dsub costs that pipe one product a row and not one
+// addition a flip.  FP64, in turn and now (us): 4x5 lattice, one column 55 and
+// 33, two 76 and 50; 22-site ladder, one 104 and 69; 4x6 lattice, two 1066 and
+// 706, eight 3058 and 2356 (2612 without the integers).  FP32, 22-site ladder,
+// eight columns 175 -> 105.  One target at a time or four cost more (4x6
+// lattice, eight 2586; 4x5, two 61).  Narrower FP32 rows take every bond in
+// turn: the test is most of their work (22-site ladder, two FP32 columns: 52 us
+// in turn, 66 us walked), and the integers cost them more than they save
+// (FP64 in turn with them: 4x5 lattice 57 against 55).
+template <typename T, int NV>
+constexpr bool kWalkRow = sizeof(T) == 8 || NV * sizeof(T) >= 32;
+
+template <typename T, int NV, bool COHERENT, bool VEC, bool WALK = kWalkRow<T, NV>>
 __device__ __forceinline__ void row_flips(const U1View &u, uint64_t s, const uint64_t *sm_mask, const T *sm_half, int nb,
-                                          const T *x, T (&acc)[NV], T &dsub) {
+                                          const T *x, T (&acc)[NV], T &dsub, const long long *fix = nullptr) {
     constexpr int D = 2;
+    long long sum = 0;
     if constexpr (!WALK) {
         for (int b = 0; b < nb; ++b) {
             const uint64_t mk = sm_mask[b], t = s & mk;
@@ -160,32 +170,45 @@ __device__ __forceinline__ void row_flips(const U1View &u, uint64_t s, const uin
             while (fl) {
                 bool on[D];
                 T cf[D], xv[D][NV];
-    #pragma unroll
+#pragma unroll
                 for (int d = 0; d < D; ++d) {
                     on[d] = fl != 0;
                     if (on[d]) {
                         const int b = b0 + __ffs(fl) - 1;
                         fl &= fl - 1;
                         cf[d] = sm_half[b];
+                        if (fix) sum += fix[b];
                         load_row<T, NV, COHERENT, VEC>(x, rank_of(u, s ^ sm_mask[b]), xv[d]);
                     }
                 }
-    #pragma unroll
+#pragma unroll
                 for (int d = 0; d < D; ++d)
                     if (on[d]) {
-    #pragma unroll
+#pragma unroll
                         for (int k = 0; k < NV; ++k) acc[k] = fma_rn(cf[d], xv[d][k], acc[k]);
-                        dsub += cf[d];
+                        if (!fix) dsub += cf[d];
                     }
             }
         }
     }
+    if (WALK && fix) dsub = (T)((double)sum * __longlong_as_double(fix[nb]));
 }
 
-// Bond masks and J_b/2 from the handle's bond table [J (nb) | masks (nb) | sum J / 4].
+// FP64 rows take the integer J_b/2 in shared memory, up to this many bonds and
+// where the couplings have a unit.
+constexpr int kFixBonds = 2048;
 template <typename T>
-__device__ __forceinline__ void stage_bonds(const double *__restrict__ bond, int nb, uint64_t *sm_mask, T *sm_half) {
+constexpr bool kFixRow = sizeof(T) == 8;
+
+// Bond masks and J_b/2 from the handle's bond table [J (nb) | masks (nb) | sum
+// J / 4 | unit | J/2 in units (nb)]; sm_fix: [nb + 1], or null.
+template <typename T>
+__device__ __forceinline__ void stage_bonds(const double *__restrict__ bond, int nb, uint64_t *sm_mask, T *sm_half,
+                                            long long *sm_fix = nullptr) {
     const uint64_t *masks = (const uint64_t *)(bond + nb);
+    if (sm_fix)
+        for (int b = threadIdx.x; b <= nb; b += blockDim.x)
+            sm_fix[b] = __double_as_longlong(b < nb ? bond[2 * nb + 2 + b] : bond[2 * nb + 1]);
     for (int b = threadIdx.x; b < nb; b += blockDim.x) {
         sm_half[b] = (T)(0.5 * bond[b]);
         sm_mask[b] = masks[b];
@@ -196,7 +219,7 @@ __device__ __forceinline__ void stage_bonds(const double *__restrict__ bond, int
 // every thread of the CTA calls it (the tile unranking has barriers).
 template <typename T, int NV, bool COHERENT, bool VEC>
 __device__ __forceinline__ void apply_rows(const U1View &u, const uint64_t *sm_mask, const T *sm_half, int nb,
-                                           T jq, const T *x, T *y, uint64_t *sh_range) {
+                                           T jq, const T *x, T *y, uint64_t *sh_range, const long long *fix) {
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < u.dim; base += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = base + threadIdx.x;
         const RowState rs = unrank_tile(u, base, r, sh_range);
@@ -206,7 +229,7 @@ __device__ __forceinline__ void apply_rows(const U1View &u, const uint64_t *sm_m
 #pragma unroll
         for (int k = 0; k < NV; ++k) acc[k] = T(0);
         T dsub = T(0);
-        row_flips<T, NV, COHERENT, VEC>(u, s, sm_mask, sm_half, nb, x, acc, dsub);
+        row_flips<T, NV, COHERENT, VEC>(u, s, sm_mask, sm_half, nb, x, acc, dsub, fix);
         T xr[NV];
         load_row<T, NV, COHERENT, VEC>(x, r, xr);
         const T d = jq - dsub;
