@@ -95,7 +95,7 @@ struct AccOf<float> {
 
 // Flip tables of the cooperative Lanczos passes: 24 bits of row, 8 of bond,
 // after the bond table in shared memory.
-constexpr int kLzTabRow = 24, kLzTabBonds = 256;
+constexpr int kLzTabRow = 24, kLzTabBonds = 256, kLzTabBytes = 128 * 1024;
 template <typename T>
 __host__ __device__ inline size_t lz_tab_at(int nb) {
     return ((size_t)nb * (sizeof(uint64_t) + sizeof(T)) + 15) / 16 * 16;
@@ -625,12 +625,13 @@ static bool lz_small_shape(const xd_ham_s *h, LzSmall *out) {
     for (int tab = 1; tab >= 0; --tab) {
         if (tab && b->nb > kLzTabBonds) continue;
         const size_t smem = lz_tab_at<T>(b->nb) + (tab ? (size_t)b->nb * kThreads * sizeof(uint32_t) : 0);
-        if (smem > (tab ? 128 * 1024 : 48 * 1024)) continue;
+        if (smem > (size_t)(tab ? kLzTabBytes : 48 * 1024)) continue;
         const void *k1 = tab ? (const void *)k_lz_persist<T, true> : (const void *)k_lz_persist<T, false>;
         const void *k2 = tab ? (const void *)k_lz_persist2<T, true> : (const void *)k_lz_persist2<T, false>;
         int per1 = 0, per2 = 0;
-        if (cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-            cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        // the limit, not this block's size: another thread may be about to launch a larger one
+        if (cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, tab ? kLzTabBytes : 48 * 1024) != cudaSuccess ||
+            cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, tab ? kLzTabBytes : 48 * 1024) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per1, k1, kThreads, smem) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per2, k2, kThreads, smem) != cudaSuccess) {
             cudaGetLastError();

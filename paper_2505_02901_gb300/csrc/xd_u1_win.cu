@@ -1184,7 +1184,8 @@ static xd_status launch_passes(const xd_ham_s *h, const void *x, void *y, cudaSt
                 set_error("U(1) product: %u bytes of shared memory do not fit", o);
                 return XD_ERANGE;
             }
-            XD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)o));
+            // the limit, not this pass's size: another thread may be about to launch a larger one
+            XD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
             const int grid = d.nctas[cq];
             kern<<<grid, kT, o, st>>>(p, x, y);
             XD_CUDA(cudaGetLastError());
