@@ -257,7 +257,7 @@ def random_vector(dim: int, seed: int, dtype=torch.float64, out=None) -> torch.T
 
 
 def batch_apply(hams, xs, ys) -> None:
-    """ys[k] = H_k xs[k] for every k in one persistent, graph-replayed launch."""
+    """ys[k] = H_k xs[k] for every k in one replayed graph."""
     n = len(hams)
     if not (n == len(xs) == len(ys)) or n == 0:
         raise ValueError("hams, xs, ys must be non-empty and of equal length")

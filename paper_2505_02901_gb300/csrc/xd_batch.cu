@@ -1,5 +1,6 @@
 // xd_batch.cu -- many independent U(1) products in one call, the small ones
-// in one persistent launch (the multi-vector apply of Sec. 5.1 over a batch of blocks; a9).
+// in one persistent launch (the multi-vector apply of Sec. 5.1 over a batch of
+// blocks; a9).
 //
 // Work list: instance k owns ceil(dim_k / tile) row tiles; tile t of the
 // whole batch maps to (instance, first row) through the prefix sums
