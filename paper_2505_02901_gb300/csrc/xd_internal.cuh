@@ -151,10 +151,10 @@ struct WinPassDev {
     WinTables T;                         // the words and slot counts (the lists follow with the couplings)
     uint64_t *d_whi = nullptr, *d_ohi = nullptr, *d_olo = nullptr;
     uint32_t *d_olo_off = nullptr;
-    WinSeg *d_segs[5] = {};              // tiles of 1, 2, 4, 8, 16 columns
-    WinCta *d_ctas[5] = {};              // their division among the CTAs
-    WinRun *d_runs[5] = {};
-    int nseg[5] = {}, nctas[5] = {}, nbase[5] = {};
+    WinSeg *d_segs[kWinForms] = {};      // tiles of kWinCols columns
+    WinCta *d_ctas[kWinForms] = {};      // their division among the CTAs
+    WinRun *d_runs[kWinForms] = {};
+    int nseg[kWinForms] = {}, nctas[kWinForms] = {}, nbase[kWinForms] = {};
 };
 
 struct WinLayoutHost {

@@ -879,7 +879,6 @@ __global__ void __launch_bounds__(kT, 1) k_win(const __grid_constant__ WinParams
 
 // ------------------------------------------------------------ host side
 constexpr uint32_t kMaxSmem = 225 * 1024;  // of the 227 KB a CTA can have; the kernel keeps 1.3 KB of its own
-constexpr int kCo = 5;  // column counts 1, 2, 4, 8, 16
 
 // Tables gathered on the host for one allocation and one copy.
 struct Pack {
@@ -921,11 +920,11 @@ xd_status win_layout_build(xd_basis_s *b) {
         pack.add(&d.d_olo, d.T.olo);
         pack.add(&d.d_olo_off, d.T.olo_off);
         pack.add(&d.d_whi, d.T.whi);
-        for (int q = 0; q < kCo; ++q) {
+        for (int q = 0; q < kWinForms; ++q) {
             int64_t nitems = 0;
             std::vector<WinCta> ctas;
             std::vector<WinRun> runs;
-            const std::vector<WinSeg> segs = win_segments(p, d.T, b->nup, 1 << q, g_num_sms, &nitems, &d.nbase[q]);
+            const std::vector<WinSeg> segs = win_segments(p, d.T, b->nup, kWinCols[q], g_num_sms, &nitems, &d.nbase[q]);
             win_divide(p, d.T, segs, nitems, g_num_sms, &ctas, &runs);
             d.nseg[q] = (int)segs.size();
             d.nctas[q] = (int)ctas.size() - 1;
@@ -1126,9 +1125,11 @@ template <bool F64, int NVS>
 static xd_status launch_passes(const xd_ham_s *h, const void *x, void *y, cudaStream_t st) {
     const xd_basis_s *b = h->b;
     const WinLayoutHost &wl = b->win;
-    const int VB = F64 ? 8 : 4, co = (64 / VB) >> NVS;
-    int cq = 0;
-    while ((1 << cq) < co) ++cq;
+    constexpr WinForm form = F64 ? kWinF64 : NVS ? kWinF32x8 : kWinF32;
+    constexpr int co = kWinCols[form];
+    static_assert(co == (64 / (F64 ? 8 : 4)) >> NVS, "64 bytes to a row of a tile");
+    int cos = 0;
+    while ((1 << cos) < co) ++cos;
     const bool wide = b->dim_u1 >= (int64_t)0xffffffffll;
     for (size_t ip = 0; ip < wl.pass.size(); ++ip) {
         const WinPassDev &d = wl.pass[ip];
@@ -1139,13 +1140,13 @@ static xd_status launch_passes(const xd_ham_s *h, const void *x, void *y, cudaSt
         p.L = b->L;
         p.lomask = (uint32_t)((1ull << b->L) - 1);
         p.ks = (const WinK *)(w.buf + w.oks);
-        p.segs = d.d_segs[cq];
-        p.nseg = d.nseg[cq];
-        p.ctas = d.d_ctas[cq];
-        p.runs = d.d_runs[cq];
+        p.segs = d.d_segs[form];
+        p.nseg = d.nseg[form];
+        p.ctas = d.d_ctas[form];
+        p.runs = d.d_runs[form];
         p.c0 = d.p.c0;
         p.co = co;
-        p.cos = cq;
+        p.cos = cos;
         p.slot_dep = (const uint64_t *)(w.buf + w.osd);
         p.ohi = d.d_ohi;
         p.olo = d.d_olo;
@@ -1176,7 +1177,7 @@ static xd_status launch_passes(const xd_ham_s *h, const void *x, void *y, cudaSt
         p.sm_step = take((size_t)w.maxstep * 8);
         p.sm_coef = take((size_t)w.ncoef * 8);
         p.sm_rinfo = take(d.p.rows ? kWinSlots * 4 : 0);
-        p.base_bytes = (uint32_t)(((size_t)d.nbase[cq] * (wide ? 8 : 4) + 15) / 16 * 16);
+        p.base_bytes = (uint32_t)(((size_t)d.nbase[form] * (wide ? 8 : 4) + 15) / 16 * 16);
         p.nbase_bufs = o + 3 * p.base_bytes <= kMaxSmem ? 3 : 2;
         p.sm_base = take((size_t)p.nbase_bufs * p.base_bytes);
         auto go = [&](auto kern) -> xd_status {
@@ -1186,7 +1187,7 @@ static xd_status launch_passes(const xd_ham_s *h, const void *x, void *y, cudaSt
             }
             // the limit, not this pass's size: another thread may be about to launch a larger one
             XD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
-            const int grid = d.nctas[cq];
+            const int grid = d.nctas[form];
             kern<<<grid, kT, o, st>>>(p, x, y);
             XD_CUDA(cudaGetLastError());
             return XD_OK;

@@ -42,6 +42,11 @@ constexpr int kWinLow = 4;       // the sites that are in a window together
 constexpr int kWinMaxBonds = 63; // bonds of a pass (6 bits of a list entry, one value left for padding)
 constexpr int kWinMaxGroups = 4; // couplings of a pass whose flips are listed coupling by coupling
 constexpr int kWinSlots = 1024;  // most row slots of a tile, its zero rows included
+// The value types of a product, and the columns of their tiles: 64 bytes of
+// values under one window word, a column being one word o (eight values of it in
+// the last).
+enum WinForm { kWinF64, kWinF32, kWinF32x8, kWinForms };
+constexpr int kWinCols[kWinForms] = {8, 16, 2};
 constexpr int kWinRows = 16;     // rows of a warp step: two to each lane of four that share a row's columns
 
 struct WinPass {
