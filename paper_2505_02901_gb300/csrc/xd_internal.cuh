@@ -241,6 +241,7 @@ struct xd_ham_s {
     // (xd_u1_win.cu): fixed point when the couplings are small integer
     // multiples of one quantum, else double-float
     std::vector<xd::WinPassHam> win;
+    bool win_fit[xd::kWinForms] = {};  // every pass fits in shared memory for products of this value type
     bool x64_fx_ok = false;         // the couplings have a quantum: fixed point allowed
     double x64_qs = 1.0;
     int x64_B = 0;
@@ -301,7 +302,7 @@ xd_status spmm_layout_build(xd_basis_s *b);
 void spmm_layout_free(xd_basis_s *b);
 xd_status spmm_ham_tables(xd_ham_s *h);
 // product in passes over windows of sites (xd_u1_win.cu): FP64 in fixed point
-// or double-float, FP32
+// or double-float, FP32; for the value types whose win_fit is set
 bool win_layout_wanted(const xd_basis_s *b);
 xd_status win_layout_build(xd_basis_s *b);
 void win_layout_free(xd_basis_s *b);

@@ -228,17 +228,17 @@ xd_status u1_states(const xd_basis_s *b, int64_t first, int64_t count, uint64_t 
 
 xd_status u1_apply(const xd_ham_s *h, const void *x, void *y, xd_dtype dt, int nvec,
                    cudaStream_t st) {
-    if (nvec == 1 && dt == XD_F32 && h->b->win.spmm32) return spmm_apply(h, x, y, st);
-    if (nvec == 1 && h->b->win.ok) {
-        xd_status s = dt == XD_F64 && passes_wanted(h->b) ? passes_apply_f64(h, x, y, st) : XD_ERANGE;
-        if (s == XD_ERANGE) s = dt == XD_F64 ? win_apply_f64(h, x, y, st) : win_apply_f32(h, x, y, st);
-        // an FP64 workspace or tables (very dense graphs) that do not fit send this product to the block kernel
+    // window tables that do not fit in shared memory (very dense graphs) leave the
+    // products to the kernels below, before anything is launched
+    if (nvec == 1 && dt == XD_F32 && h->b->spmm.ok && (h->b->win.spmm32 || !h->win_fit[kWinF32])) return spmm_apply(h, x, y, st);
+    if (nvec == 1 && dt == XD_F32 && h->win_fit[kWinF32]) return win_apply_f32(h, x, y, st);
+    if (nvec == 1 && dt == XD_F64 && h->b->win.ok) {
+        xd_status s = passes_wanted(h->b) ? passes_apply_f64(h, x, y, st) : XD_ERANGE;
+        if (s == XD_ERANGE && h->win_fit[kWinF64]) s = win_apply_f64(h, x, y, st);
+        // a workspace that does not fit sends this product to the block kernel
         if (s != XD_ENOMEM && s != XD_ERANGE) return s;
     }
-    if (nvec == 8 && dt == XD_F32 && win8_usable(h, x, y)) {
-        const xd_status s = win8_apply(h, x, y, st);
-        if (s != XD_ERANGE) return s;
-    }
+    if (nvec == 8 && dt == XD_F32 && win8_usable(h, x, y)) return win8_apply(h, x, y, st);
     if (nvec == 8 && dt == XD_F32 && spmm8_usable(h, x, y)) return spmm8_apply(h, x, y, st);
     if (nvec == 1 && h->b->blk.ok) return block_apply(h, x, y, dt, st);
     if (dt == XD_F64) {

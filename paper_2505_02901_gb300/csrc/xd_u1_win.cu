@@ -878,7 +878,6 @@ __global__ void __launch_bounds__(kT, 1) k_win(const __grid_constant__ WinParams
 }  // namespace
 
 // ------------------------------------------------------------ host side
-constexpr uint32_t kMaxSmem = 225 * 1024;  // of the 227 KB a CTA can have; the kernel keeps 1.3 KB of its own
 
 // Tables gathered on the host for one allocation and one copy.
 struct Pack {
@@ -898,6 +897,9 @@ struct Pack {
         return XD_OK;
     }
 };
+
+// 64-bit row offsets
+static bool win_wide(const xd_basis_s *b) { return b->dim_u1 >= (int64_t)0xffffffffll; }
 
 bool win_layout_wanted(const xd_basis_s *b) { return !b->sym && b->N >= 24; }
 
@@ -972,7 +974,9 @@ xd_status win_ham_tables(xd_ham_s *h) {
     while ((int64_t(1) << lg) < 3 * std::max<int64_t>(1, kabs)) ++lg;
     h->x64_B = 62 - lg;
     h->x64_qs = 0.25 * q;
+    const bool wide = win_wide(b);
     h->win.resize(wl.pass.size());
+    std::fill(h->win_fit, h->win_fit + kWinForms, true);
     for (size_t ip = 0; ip < wl.pass.size(); ++ip) {
         const WinPassDev &pd = wl.pass[ip];
         WinPassHam &w = h->win[ip];
@@ -1079,6 +1083,9 @@ xd_status win_ham_tables(xd_ham_s *h) {
             d2[s] = (float)Dj[v];
         }
         XD_CUDA(cudaMemcpy(w.buf + w.ovar, var.data(), var.size(), cudaMemcpyHostToDevice));
+        for (int f = 0; f < kWinForms; ++f)
+            h->win_fit[f] = h->win_fit[f] &&
+                            win_smem(p.rows, w.maxslots, w.maxlist, w.maxstep, w.ncoef, pd.nbase[f], wide).fits();
     }
     return XD_OK;
 }
@@ -1120,7 +1127,7 @@ void x64_release(xd_ham_s *h) {
     }
 }
 
-// The passes; NVS = log2 of the vectors per row: 0, or 3 in FP32.
+// The passes (win_fit is set); NVS = log2 of the vectors per row: 0, or 3 in FP32.
 template <bool F64, int NVS>
 static xd_status launch_passes(const xd_ham_s *h, const void *x, void *y, cudaStream_t st) {
     const xd_basis_s *b = h->b;
@@ -1130,7 +1137,7 @@ static xd_status launch_passes(const xd_ham_s *h, const void *x, void *y, cudaSt
     static_assert(co == (64 / (F64 ? 8 : 4)) >> NVS, "64 bytes to a row of a tile");
     int cos = 0;
     while ((1 << cos) < co) ++cos;
-    const bool wide = b->dim_u1 >= (int64_t)0xffffffffll;
+    const bool wide = win_wide(b);
     for (size_t ip = 0; ip < wl.pass.size(); ++ip) {
         const WinPassDev &d = wl.pass[ip];
         const WinPassHam &w = h->win[ip];
@@ -1166,29 +1173,20 @@ static xd_status launch_passes(const xd_ham_s *h, const void *x, void *y, cudaSt
         p.qs = h->x64_qs;
         p.B = h->x64_B;
         p.state = h->d_x64_state;
-        uint32_t o = (uint32_t)w.maxslots * 128;
-        p.sm_tile1 = (uint32_t)w.maxslots * 64;
-        auto take = [&](size_t bytes) {
-            const uint32_t at = o;
-            o += (uint32_t)((bytes + 15) / 16 * 16);
-            return at;
-        };
-        p.sm_list = take((size_t)w.maxlist * 4);
-        p.sm_step = take((size_t)w.maxstep * 8);
-        p.sm_coef = take((size_t)w.ncoef * 8);
-        p.sm_rinfo = take(d.p.rows ? kWinSlots * 4 : 0);
-        p.base_bytes = (uint32_t)(((size_t)d.nbase[form] * (wide ? 8 : 4) + 15) / 16 * 16);
-        p.nbase_bufs = o + 3 * p.base_bytes <= kMaxSmem ? 3 : 2;
-        p.sm_base = take((size_t)p.nbase_bufs * p.base_bytes);
+        const WinSmem sm = win_smem(d.p.rows, w.maxslots, w.maxlist, w.maxstep, w.ncoef, d.nbase[form], wide);
+        p.sm_tile1 = sm.tile1;
+        p.sm_list = sm.list;
+        p.sm_step = sm.step;
+        p.sm_coef = sm.coef;
+        p.sm_rinfo = sm.rinfo;
+        p.base_bytes = sm.base_bytes;
+        p.nbase_bufs = sm.base_sets;
+        p.sm_base = sm.base;
         auto go = [&](auto kern) -> xd_status {
-            if (o > kMaxSmem) {
-                set_error("U(1) product: %u bytes of shared memory do not fit", o);
-                return XD_ERANGE;
-            }
             // the limit, not this pass's size: another thread may be about to launch a larger one
-            XD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
+            XD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWinSmem));
             const int grid = d.nctas[form];
-            kern<<<grid, kT, o, st>>>(p, x, y);
+            kern<<<grid, kT, sm.total, st>>>(p, x, y);
             XD_CUDA(cudaGetLastError());
             return XD_OK;
         };
@@ -1197,7 +1195,8 @@ static xd_status launch_passes(const xd_ham_s *h, const void *x, void *y, cudaSt
             if (d.p.rows) return p.ng ? go(k_win<F64, true, false, NVS, I>) : go(k_win<F64, true, true, NVS, I>);
             return p.ng ? go(k_win<F64, false, false, NVS, I>) : go(k_win<F64, false, true, NVS, I>);
         };
-        XD_TRY(wide ? pick((unsigned long long)0) : pick((unsigned)0));
+        if constexpr (NVS == 0) XD_TRY(wide ? pick((unsigned long long)0) : pick((unsigned)0));
+        else XD_TRY(pick((unsigned)0));  // win8_usable: no 64-bit row offsets
     }
     return XD_OK;
 }
@@ -1222,11 +1221,11 @@ xd_status win_apply_f32(const xd_ham_s *h, const void *x, void *y, cudaStream_t 
 // 28000 and 3600 a flip, bonds listed twice counted twice).  Measured, here
 // and there (us): 28-site ladder 3843 and 6545, 4x7 lattice 5649 and 8507,
 // 24-site ladder 320 and 375; 28-site chain 3527 and 2572, 24-site chain 276
-// and 154.  The dimension keeps every table inside shared memory (32-bit row
-// offsets).
+// and 154.  Where the tables of a pass do not fit, and where row offsets have 64
+// bits, the prefix blocks stay.
 bool win8_usable(const xd_ham_s *h, const void *x, const void *y) {
     const xd_basis_s *b = h->b;
-    return b->win.ok && b->dim_u1 < (int64_t)0xffffffffll && (((uintptr_t)x | (uintptr_t)y) & 15) == 0 &&
+    return h->win_fit[kWinF32x8] && !win_wide(b) && (((uintptr_t)x | (uintptr_t)y) & 15) == 0 &&
            26000.0 * b->win.pass.size() + 700.0 * win_flips(b->N, b->nup, (int)b->win.pairs.size()) <
                28000.0 + 3600.0 * win_flips(b->N, b->nup, b->nb);
 }

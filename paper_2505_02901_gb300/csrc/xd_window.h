@@ -679,6 +679,38 @@ inline std::vector<WinSeg> win_segments(const WinPass &p, const WinTables &T, in
     return out;
 }
 
+// The shared memory of a CTA: two tiles, the flip lists and step headers of one
+// popcount, the coefficients, (rows kind) the rows, and three sets of row
+// offsets, or two where three do not fit.  T: maxslots, maxlist, maxstep; nbase:
+// of win_segments; wide: 64-bit row offsets.
+constexpr uint32_t kWinSmem = 225 * 1024;  // of the 227 KB a CTA can have; the kernel keeps 1.3 KB of its own
+
+struct WinSmem {
+    uint32_t tile1, list, step, coef, rinfo, base, base_bytes, total;
+    int base_sets;
+    bool fits() const { return total <= kWinSmem; }
+};
+
+inline WinSmem win_smem(bool rows, int maxslots, int maxlist, int maxstep, int ncoef, int nbase, bool wide) {
+    WinSmem s{};
+    uint32_t o = (uint32_t)maxslots * 128;
+    auto take = [&](size_t bytes) {
+        const uint32_t at = o;
+        o += (uint32_t)((bytes + 15) / 16 * 16);
+        return at;
+    };
+    s.tile1 = (uint32_t)maxslots * 64;
+    s.list = take((size_t)maxlist * 4);
+    s.step = take((size_t)maxstep * 8);
+    s.coef = take((size_t)ncoef * 8);
+    s.rinfo = take(rows ? kWinSlots * 4 : 0);
+    s.base_bytes = (uint32_t)(((size_t)nbase * (wide ? 8 : 4) + 15) / 16 * 16);
+    s.base_sets = o + 3 * s.base_bytes <= kWinSmem ? 3 : 2;
+    s.base = take((size_t)s.base_sets * s.base_bytes);
+    s.total = o;
+    return s;
+}
+
 // The tiles' division among at most `ctas` CTAs.  Many tiles (kWinMany to a
 // CTA): a run of every popcount k, of equal length up to one, the longer ones
 // dealt on from k to k; all CTAs then work on tiles of one cost at a time.
