@@ -148,7 +148,6 @@ struct PassLayoutHost {
 // The window passes of a large U(1) block (xd_u1_win.cu).
 struct WinPassDev {
     WinPass p;
-    WinTables T;                         // the words and slot counts (the lists follow with the couplings)
     uint64_t *d_whi = nullptr, *d_ohi = nullptr, *d_olo = nullptr;
     uint32_t *d_olo_off = nullptr;
     WinSeg *d_segs[kWinForms] = {};      // tiles of kWinCols columns
@@ -171,7 +170,9 @@ struct WinPassHam {
     unsigned char *buf = nullptr;
     size_t cap = 0, bytes = 0, oks = 0, osd = 0, ori = 0, oli = 0, ost = 0, ovar = 0;
     size_t oc[3] = {}, od[3] = {};       // double-float, fixed point, FP32
+    int groups = -1;                     // wanted coupling groups (0: the bond in each entry)
     int ng = -1, ncoef = 0, maxslots = 0, maxlist = 0, maxstep = 0;
+    bool fit[kWinForms] = {};
     std::vector<int> gid;                // coupling group of every bond of the pass
     std::vector<uint16_t> slot_word;
 };

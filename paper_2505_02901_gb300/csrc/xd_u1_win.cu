@@ -898,9 +898,6 @@ struct Pack {
     }
 };
 
-// 64-bit row offsets
-static bool win_wide(const xd_basis_s *b) { return b->dim_u1 >= (int64_t)0xffffffffll; }
-
 bool win_layout_wanted(const xd_basis_s *b) { return !b->sym && b->N >= 24; }
 
 // The passes of the block's graph, the words outside their windows and the
@@ -909,32 +906,25 @@ xd_status win_layout_build(xd_basis_s *b) {
     WinLayoutHost &wl = b->win;
     grid_for(1, 1, 1);
     wl.pairs = win_pairs((const int32_t *)b->bonds.data(), b->nb, &wl.pair_of);
-    const std::vector<WinPass> passes = choose_windows(b->N, b->nup, wl.pairs);
-    wl.pass.resize(passes.size());
+    const std::vector<WinPlan> plan = win_plan(b->N, b->nup, wl.pairs, g_num_sms);
+    wl.pass.resize(plan.size());
     Pack pack;
-    for (size_t ip = 0; ip < passes.size(); ++ip) {
-        const WinPass &p = passes[ip];
+    for (size_t ip = 0; ip < plan.size(); ++ip) {
+        const WinPlan &s = plan[ip];
         WinPassDev &d = wl.pass[ip];
-        d.p = p;
-        win_shape(p, win_classes(p, wl.pairs), &d.T);
-        win_outer(p, b->nup, &d.T);
-        pack.add(&d.d_ohi, d.T.ohi);
-        pack.add(&d.d_olo, d.T.olo);
-        pack.add(&d.d_olo_off, d.T.olo_off);
-        pack.add(&d.d_whi, d.T.whi);
+        d.p = s.p;
+        pack.add(&d.d_ohi, s.T.ohi);
+        pack.add(&d.d_olo, s.T.olo);
+        pack.add(&d.d_olo_off, s.T.olo_off);
+        pack.add(&d.d_whi, s.T.whi);
         for (int q = 0; q < kWinForms; ++q) {
-            int64_t nitems = 0;
-            std::vector<WinCta> ctas;
-            std::vector<WinRun> runs;
-            const std::vector<WinSeg> segs = win_segments(p, d.T, b->nup, kWinCols[q], g_num_sms, &nitems, &d.nbase[q]);
-            win_divide(p, d.T, segs, nitems, g_num_sms, &ctas, &runs);
-            d.nseg[q] = (int)segs.size();
-            d.nctas[q] = (int)ctas.size() - 1;
-            pack.add(&d.d_segs[q], segs);
-            pack.add(&d.d_ctas[q], ctas);
-            pack.add(&d.d_runs[q], runs);
+            d.nseg[q] = (int)s.segs[q].size();
+            d.nctas[q] = (int)s.ctas[q].size() - 1;
+            d.nbase[q] = s.nbase[q];
+            pack.add(&d.d_segs[q], s.segs[q]);
+            pack.add(&d.d_ctas[q], s.ctas[q]);
+            pack.add(&d.d_runs[q], s.runs[q]);
         }
-        d.T.ohi = d.T.olo = std::vector<uint64_t>();  // on the device only from here on
     }
     XD_TRY(pack.upload(&wl.buf));
     wl.spmm32 = spmm_better(b);
@@ -950,8 +940,9 @@ void win_layout_free(xd_basis_s *b) {
 // Flip lists, coefficients and diagonals of every pass.  Flips are listed
 // coupling by coupling when a pass has at most kWinMaxGroups of them (one
 // multiplication per row and coupling; measured at the 4x8 J1-J2 lattice
-// against entries that carry their bond), else with the bond in each entry.
-// The lists are made again only when the pattern of equal couplings changes.
+// against entries that carry their bond) and they fit (win_fitting_lists),
+// else with the bond in each entry.  The lists are made again only when the
+// pattern of equal couplings changes.
 xd_status win_ham_tables(xd_ham_s *h) {
     const xd_basis_s *b = h->b;
     const WinLayoutHost &wl = b->win;
@@ -974,7 +965,7 @@ xd_status win_ham_tables(xd_ham_s *h) {
     while ((int64_t(1) << lg) < 3 * std::max<int64_t>(1, kabs)) ++lg;
     h->x64_B = 62 - lg;
     h->x64_qs = 0.25 * q;
-    const bool wide = win_wide(b);
+    const bool wide = win_wide(b->dim_u1);
     h->win.resize(wl.pass.size());
     std::fill(h->win_fit, h->win_fit + kWinForms, true);
     for (size_t ip = 0; ip < wl.pass.size(); ++ip) {
@@ -989,15 +980,15 @@ xd_status win_ham_tables(xd_ham_s *h) {
             gid[t] = (int)(std::find(vals.begin(), vals.end(), v) - vals.begin());
             if (gid[t] == (int)vals.size()) vals.push_back(v);
         }
-        const int ng = (int)vals.size() <= kWinMaxGroups ? (int)vals.size() : 0;
-        if (!ng) gid.assign(nwb, 0);
-        const bool fresh = !w.buf || w.ng != ng || w.gid != gid;
-        const int ncoef = ng ? ng : kWinMaxBonds + 1;
+        const int groups = (int)vals.size() <= kWinMaxGroups ? (int)vals.size() : 0;
+        if (!groups) gid.assign(nwb, 0);
+        const bool fresh = !w.buf || w.groups != groups || w.gid != gid;
         auto up16 = [](size_t v) { return (v + 15) / 16 * 16; };
         if (fresh) {
             WinTables T;
-            win_lists(p, wl.pairs, gid, ng, &T);
-            w.ng = ng;
+            w.ng = win_fitting_lists(p, wl.pairs, pd.nbase, wide, gid, groups, &T, w.fit);
+            w.ncoef = w.ng ? w.ng : kWinMaxBonds + 1;
+            w.groups = groups;
             w.gid = gid;
             w.slot_word = T.slot_word;
             w.maxslots = T.maxslots;
@@ -1045,7 +1036,6 @@ xd_status win_ham_tables(xd_ham_s *h) {
                 w.od[a] = od[a];
             }
         }
-        w.ncoef = ncoef;
         // coefficients (double-float, fixed point, FP32) and the window words' diagonals
         auto pair = [](double d) {
             const float c = (float)d;
@@ -1059,7 +1049,7 @@ xd_status win_ham_tables(xd_ham_s *h) {
         std::vector<int> Dk(1u << ws, 0);
         for (int t = 0; t < nwb; ++t) {
             const auto &pr = wl.pairs[p.bonds[t]];
-            const int at = ng ? gid[t] : t, kb = kp[p.bonds[t]];
+            const int at = w.ng ? gid[t] : t, kb = kp[p.bonds[t]];
             const double j = Jp[p.bonds[t]];
             c0[at] = pair(0.5 * j);
             c1[at] = 2 * kb;
@@ -1083,9 +1073,7 @@ xd_status win_ham_tables(xd_ham_s *h) {
             d2[s] = (float)Dj[v];
         }
         XD_CUDA(cudaMemcpy(w.buf + w.ovar, var.data(), var.size(), cudaMemcpyHostToDevice));
-        for (int f = 0; f < kWinForms; ++f)
-            h->win_fit[f] = h->win_fit[f] &&
-                            win_smem(p.rows, w.maxslots, w.maxlist, w.maxstep, w.ncoef, pd.nbase[f], wide).fits();
+        for (int f = 0; f < kWinForms; ++f) h->win_fit[f] = h->win_fit[f] && w.fit[f];
     }
     return XD_OK;
 }
@@ -1137,7 +1125,7 @@ static xd_status launch_passes(const xd_ham_s *h, const void *x, void *y, cudaSt
     static_assert(co == (64 / (F64 ? 8 : 4)) >> NVS, "64 bytes to a row of a tile");
     int cos = 0;
     while ((1 << cos) < co) ++cos;
-    const bool wide = win_wide(b);
+    const bool wide = win_wide(b->dim_u1);
     for (size_t ip = 0; ip < wl.pass.size(); ++ip) {
         const WinPassDev &d = wl.pass[ip];
         const WinPassHam &w = h->win[ip];
@@ -1225,7 +1213,7 @@ xd_status win_apply_f32(const xd_ham_s *h, const void *x, void *y, cudaStream_t 
 // bits, the prefix blocks stay.
 bool win8_usable(const xd_ham_s *h, const void *x, const void *y) {
     const xd_basis_s *b = h->b;
-    return h->win_fit[kWinF32x8] && !win_wide(b) && (((uintptr_t)x | (uintptr_t)y) & 15) == 0 &&
+    return h->win_fit[kWinF32x8] && (((uintptr_t)x | (uintptr_t)y) & 15) == 0 &&
            26000.0 * b->win.pass.size() + 700.0 * win_flips(b->N, b->nup, (int)b->win.pairs.size()) <
                28000.0 + 3600.0 * win_flips(b->N, b->nup, b->nb);
 }

@@ -679,6 +679,9 @@ inline std::vector<WinSeg> win_segments(const WinPass &p, const WinTables &T, in
     return out;
 }
 
+// 64-bit row offsets
+inline bool win_wide(int64_t dim) { return dim >= (int64_t)0xffffffffll; }
+
 // The shared memory of a CTA: two tiles, the flip lists and step headers of one
 // popcount, the coefficients, (rows kind) the rows, and three sets of row
 // offsets, or two where three do not fit.  T: maxslots, maxlist, maxstep; nbase:
@@ -773,6 +776,91 @@ inline void win_divide(const WinPass &p, const WinTables &T, const std::vector<W
         }
     }
     (*cta)[n].run0 = (int32_t)runs->size();
+}
+
+// Flip lists of a pass with bonds in ng coupling groups (gid): coupling by
+// coupling, or with the bond in each entry (ng = 0).  Every coupling pads its
+// part of a step's lists, so that with several of them on a dense graph the
+// lists coupling by coupling may not fit in shared memory; the pass then takes
+// the entries that carry the bond where these leave room for more value types
+// (lists of 63 bonds and four couplings: 96 KB and 72 KB).  Returns the ng
+// taken; fit: whether products of each value type fit (64-bit row offsets: none
+// on eight vectors).
+inline int win_fitting_lists(const WinPass &p, const std::vector<std::pair<int, int>> &pairs, const int *nbase, bool wide,
+                             const std::vector<int> &gid, int ng, WinTables *T, bool *fit) {
+    auto room = [&](const WinTables &t, int groups, bool *f) {
+        int n = 0;
+        for (int q = 0; q < kWinForms; ++q) {
+            f[q] = !(wide && q == kWinF32x8) &&
+                   win_smem(p.rows, t.maxslots, t.maxlist, t.maxstep, groups ? groups : kWinMaxBonds + 1, nbase[q], wide).fits();
+            n += f[q];
+        }
+        return n;
+    };
+    win_lists(p, pairs, gid, ng, T);
+    const int n = room(*T, ng, fit);
+    if (ng == 0 || n == (wide ? kWinForms - 1 : (int)kWinForms)) return ng;
+    WinTables B;
+    bool fb[kWinForms];
+    win_lists(p, pairs, std::vector<int>(p.bonds.size(), 0), 0, &B);
+    if (room(B, 0, fb) <= n) return ng;
+    *T = std::move(B);
+    std::copy(fb, fb + kWinForms, fit);
+    return 0;
+}
+
+// A pass with what does not depend on the couplings: its shape, the words
+// outside its window and, for every value type, its tiles and their division.
+struct WinPlan {
+    WinPass p;
+    WinTables T;
+    std::vector<WinSeg> segs[kWinForms];
+    std::vector<WinCta> ctas[kWinForms];
+    std::vector<WinRun> runs[kWinForms];
+    int nbase[kWinForms] = {};
+};
+
+// The passes of a block on a chip of `sms` CTAs.  A pass whose bond-carrying
+// lists would not fit is done in two, each with half of its bonds; FP32 beside
+// 64-bit row offsets (twice the room, and twice the columns of FP64) may be
+// left without.
+inline std::vector<WinPlan> win_plan(int N, int nup, const std::vector<std::pair<int, int>> &pairs, int sms) {
+    const bool wide = win_wide(n_choose_k(N, nup));
+    std::vector<WinPlan> out;
+    std::vector<WinPass> todo = choose_windows(N, nup, pairs);
+    std::reverse(todo.begin(), todo.end());
+    while (!todo.empty()) {
+        WinPlan d;
+        d.p = todo.back();
+        todo.pop_back();
+        const WinPass &p = d.p;
+        win_shape(p, win_classes(p, pairs), &d.T);
+        win_outer(p, nup, &d.T);
+        for (int q = 0; q < kWinForms; ++q) {
+            int64_t nitems = 0;
+            d.segs[q] = win_segments(p, d.T, nup, kWinCols[q], sms, &nitems, &d.nbase[q]);
+            win_divide(p, d.T, d.segs[q], nitems, sms, &d.ctas[q], &d.runs[q]);
+        }
+        // a list holds at most every bond of the pass: most passes fit at that size
+        const int nwb = (int)p.bonds.size(), most = d.T.maxstep * 2 * kWinRows * ((nwb + 3) / 4);
+        bool fit[kWinForms], all = true;
+        for (int q = 0; q < kWinForms; ++q)
+            all = all && win_smem(p.rows, d.T.maxslots, most, d.T.maxstep, kWinMaxBonds + 1, d.nbase[q], wide).fits();
+        if (!all && nwb > 1) {
+            WinTables T;
+            win_fitting_lists(p, pairs, d.nbase, wide, std::vector<int>(nwb, 0), 0, &T, fit);
+            if (wide ? !fit[kWinF64] : !(fit[kWinF64] && fit[kWinF32] && fit[kWinF32x8])) {
+                WinPass a = p, b = p;
+                a.bonds.resize(nwb / 2);
+                b.bonds.erase(b.bonds.begin(), b.bonds.begin() + nwb / 2);
+                todo.push_back(b);
+                todo.push_back(a);
+                continue;
+            }
+        }
+        out.push_back(std::move(d));
+    }
+    return out;
 }
 
 }  // namespace xd
