@@ -126,7 +126,8 @@ void xd_basis_destroy(xd_basis b);
  * symmetric block the couplings must be invariant under the group. */
 xd_status xd_ham_create(xd_basis b, const double *J, xd_ham *out);
 
-/* Replace the couplings (same validation as create). */
+/* Replace the couplings (same validation as create).  Without the memory for
+ * them (XD_ENOMEM) the handle keeps those it has. */
 xd_status xd_ham_set_couplings(xd_ham h, const double *J);
 
 void xd_ham_destroy(xd_ham h);

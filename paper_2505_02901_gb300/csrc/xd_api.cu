@@ -459,6 +459,18 @@ static xd_status set_J(xd_ham_s *h, const double *J) {
             return XD_ESYM;
         }
     }
+    // what can fail for want of memory on a handle in use comes before any change of it
+    struct Lists {
+        std::vector<WinPassHam> of;
+        ~Lists() {
+            for (WinPassHam &w : of) cudaFree(w.buf);
+        }
+    } lists;
+    if (b->win.ok) XD_TRY(win_ham_lists(h, J, &lists.of));
+    if (b->sym && !h->d_symtab) XD_TRY(sym_ham_tables(h));
+    if (b->sym) XD_TRY(sym_bond_groups(h, J));
+    lanczos_forget(h, false);
+    batch_forget(h);  // captured launches hold per-coupling scalars and addresses
     h->J.assign(J, J + b->nb);
     XD_CUDA(cudaMemcpy(h->d_J, J, sizeof(double) * b->nb, cudaMemcpyHostToDevice));
     std::vector<double> buf(3 * b->nb + 2);
@@ -482,14 +494,10 @@ static xd_status set_J(xd_ham_s *h, const double *J) {
         memcpy(&buf[2 * b->nb + 2 + k], &f, sizeof f);
     }
     XD_CUDA(cudaMemcpy(h->d_bond, buf.data(), sizeof(double) * buf.size(), cudaMemcpyHostToDevice));
-    if (b->sym && !h->d_symtab) XD_TRY(sym_ham_tables(h));
-    if (b->sym) XD_TRY(sym_bond_groups(h));
     if (b->blk.ok) XD_TRY(block_ham_tables(h));
     if (b->spmm.ok) XD_TRY(spmm_ham_tables(h));
-    if (b->win.ok) XD_TRY(win_ham_tables(h));
+    if (b->win.ok) XD_TRY(win_ham_tables(h, &lists.of));
     if (passes_wanted(b)) XD_TRY(passes_tables(h));
-    lanczos_forget(h, false);
-    batch_forget(h);  // captured batched launches hold per-coupling scalars
     return XD_OK;
 }
 

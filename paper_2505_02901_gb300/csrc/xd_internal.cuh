@@ -168,7 +168,7 @@ struct WinLayoutHost {
 // One pass's lists, coefficients and diagonals for a Hamiltonian, one allocation.
 struct WinPassHam {
     unsigned char *buf = nullptr;
-    size_t cap = 0, bytes = 0, oks = 0, osd = 0, ori = 0, oli = 0, ost = 0, ovar = 0;
+    size_t bytes = 0, oks = 0, osd = 0, ori = 0, oli = 0, ost = 0, ovar = 0;
     size_t oc[3] = {}, od[3] = {};       // double-float, fixed point, FP32
     int groups = -1;                     // wanted coupling groups (0: the bond in each entry)
     int ng = -1, ncoef = 0, maxslots = 0, maxlist = 0, maxstep = 0;
@@ -281,7 +281,7 @@ xd_status u1_bilinear_nvec(const xd_ham_s *h, const void *g, const void *x, xd_d
 // symmetric blocks (xd_sym.cu)
 xd_status sym_build(xd_basis_s *b);
 xd_status sym_ham_tables(xd_ham_s *h);
-xd_status sym_bond_groups(xd_ham_s *h);  // on every new set of couplings
+xd_status sym_bond_groups(xd_ham_s *h, const double *J);  // on every new set of couplings
 xd_status sym_apply(const xd_ham_s *h, const void *x, void *y, xd_dtype dt,
                     cudaStream_t st);
 xd_status sym_bilinear(const xd_ham_s *h, const void *g, const void *x,
@@ -307,7 +307,8 @@ xd_status spmm_ham_tables(xd_ham_s *h);
 bool win_layout_wanted(const xd_basis_s *b);
 xd_status win_layout_build(xd_basis_s *b);
 void win_layout_free(xd_basis_s *b);
-xd_status win_ham_tables(xd_ham_s *h);
+xd_status win_ham_lists(const xd_ham_s *h, const double *J, std::vector<WinPassHam> *out);
+xd_status win_ham_tables(xd_ham_s *h, std::vector<WinPassHam> *lists);
 void win_ham_free(xd_ham_s *h);
 xd_status win_apply_f64(const xd_ham_s *h, const void *x, void *y, cudaStream_t st);
 xd_status win_apply_f32(const xd_ham_s *h, const void *x, void *y, cudaStream_t st);

@@ -783,7 +783,7 @@ xd_status sym_ham_tables(xd_ham_s *h) {
     return XD_OK;
 }
 
-xd_status sym_bond_groups(xd_ham_s *h) {
+xd_status sym_bond_groups(xd_ham_s *h, const double *J) {
     const xd_basis_s *b = h->b;
     const int nb = b->nb, nchunk = (nb + 63) / 64;
     if (nb > 65535) {
@@ -792,17 +792,17 @@ xd_status sym_bond_groups(xd_ham_s *h) {
     }
     std::vector<int> order(nb);
     for (int q = 0; q < nb; ++q) order[q] = q;
-    std::stable_sort(order.begin(), order.end(), [&](int p, int q) { return h->J[p] < h->J[q]; });
+    std::stable_sort(order.begin(), order.end(), [&](int p, int q) { return J[p] < J[q]; });
     std::vector<uint64_t> gmask;
     std::vector<double> ghalf;
     std::vector<uint16_t> goff(nchunk + 1, 0);
     for (int c = 0; c < nchunk; ++c) {
         goff[c] = (uint16_t)gmask.size();
         for (int q = 64 * c; q < std::min(nb, 64 * c + 64); ++q) {
-            const double J = h->J[order[q]];
-            if (q == 64 * c || J != h->J[order[q - 1]]) {
+            const double v = J[order[q]];
+            if (q == 64 * c || v != J[order[q - 1]]) {
                 gmask.push_back(0);
-                ghalf.push_back(0.5 * J);
+                ghalf.push_back(0.5 * v);
             }
             gmask.back() |= 1ull << (q - 64 * c);
         }
@@ -819,11 +819,12 @@ xd_status sym_bond_groups(xd_ham_s *h) {
     uint16_t *u16 = (uint16_t *)(tab.data() + nb + 2 * ngrp);
     for (int q = 0; q < nb; ++q) u16[q] = (uint16_t)order[q];
     for (int c = 0; c <= nchunk; ++c) u16[nb + c] = goff[c];
-    if (h->d_symgrp && h->sym_ngrp != ngrp) {
+    if (!h->d_symgrp || h->sym_ngrp != ngrp) {  // the old table stays where the new one does not fit
+        uint64_t *grp = nullptr;
+        XD_CUDA(dev_malloc((void **)&grp, tab.size() * sizeof(uint64_t)));
         cudaFree(h->d_symgrp);
-        h->d_symgrp = nullptr;
+        h->d_symgrp = grp;
     }
-    if (!h->d_symgrp) XD_CUDA(dev_malloc((void **)&h->d_symgrp, tab.size() * sizeof(uint64_t)));
     XD_CUDA(cudaMemcpy(h->d_symgrp, tab.data(), tab.size() * sizeof(uint64_t), cudaMemcpyHostToDevice));
     h->sym_ngrp = ngrp;
     return XD_OK;

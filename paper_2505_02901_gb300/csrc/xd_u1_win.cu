@@ -937,105 +937,120 @@ void win_layout_free(xd_basis_s *b) {
     b->win = WinLayoutHost();
 }
 
-// Flip lists, coefficients and diagonals of every pass.  Flips are listed
-// coupling by coupling when a pass has at most kWinMaxGroups of them (one
-// multiplication per row and coupling; measured at the 4x8 J1-J2 lattice
-// against entries that carry their bond) and they fit (win_fitting_lists),
-// else with the bond in each entry.  The lists are made again only when the
-// pattern of equal couplings changes.
-xd_status win_ham_tables(xd_ham_s *h) {
+// The couplings of the distinct pairs.
+static std::vector<double> pair_couplings(const xd_basis_s *b, const double *J) {
+    std::vector<double> Jp(b->win.pairs.size(), 0.0);
+    for (int t = 0; t < b->nb; ++t) Jp[b->win.pair_of[t]] += J[t];
+    return Jp;
+}
+
+// Flip lists of the passes whose pattern of equal couplings is another than the
+// handle's, in new allocations (out[pass].buf; null: the handle's lists stay).
+// Flips are listed coupling by coupling when a pass has at most kWinMaxGroups of
+// them (one multiplication per row and coupling; measured at the 4x8 J1-J2
+// lattice against entries that carry their bond) and they fit
+// (win_fitting_lists), else with the bond in each entry.  Nothing of the handle
+// changes, so that an allocation that fails leaves it as it was; the caller frees
+// what is left in `out`.
+xd_status win_ham_lists(const xd_ham_s *h, const double *J, std::vector<WinPassHam> *out) {
+    const xd_basis_s *b = h->b;
+    const WinLayoutHost &wl = b->win;
+    const std::vector<double> Jp = pair_couplings(b, J);
+    const bool wide = win_wide(b->dim_u1);
+    out->assign(wl.pass.size(), WinPassHam());
+    for (size_t ip = 0; ip < wl.pass.size(); ++ip) {
+        const WinPassDev &pd = wl.pass[ip];
+        const WinPass &p = pd.p;
+        std::vector<double> vals;
+        std::vector<int> gid(p.bonds.size());
+        for (size_t t = 0; t < gid.size(); ++t) {
+            const double v = Jp[p.bonds[t]];
+            gid[t] = (int)(std::find(vals.begin(), vals.end(), v) - vals.begin());
+            if (gid[t] == (int)vals.size()) vals.push_back(v);
+        }
+        const int groups = (int)vals.size() <= kWinMaxGroups ? (int)vals.size() : 0;
+        if (!groups) std::fill(gid.begin(), gid.end(), 0);
+        if (ip < h->win.size() && h->win[ip].groups == groups && h->win[ip].gid == gid) continue;
+        WinPassHam &w = (*out)[ip];
+        WinTables T;
+        w.ng = win_fitting_lists(p, wl.pairs, pd.nbase, wide, gid, groups, &T, w.fit);
+        w.ncoef = w.ng ? w.ng : kWinMaxBonds + 1;
+        w.groups = groups;
+        w.gid = gid;
+        w.slot_word = T.slot_word;
+        w.maxslots = T.maxslots;
+        w.maxlist = T.maxlist;
+        w.maxstep = T.maxstep;
+        const size_t nslot = T.slot_word.size();
+        auto take = [&](size_t bytes) {
+            const size_t at = w.bytes;
+            w.bytes += (bytes + 15) / 16 * 16;
+            return at;
+        };
+        w.oks = take(T.k.size() * sizeof(WinK));
+        w.osd = take(nslot * 8);
+        w.ori = take(T.rinfo.size() * 4);
+        w.oli = take(T.list.size() * 4);
+        w.ost = take(T.step.size() * 4);
+        w.ovar = w.bytes;
+        const size_t cs[3] = {8, 4, 4};
+        for (int a = 0; a < 3; ++a) {
+            w.oc[a] = take((kWinMaxBonds + 1) * cs[a]);
+            w.od[a] = take(nslot * cs[a]);
+        }
+        std::vector<unsigned char> host(w.ovar, 0);
+        memcpy(&host[w.oks], T.k.data(), T.k.size() * sizeof(WinK));
+        memcpy(&host[w.osd], T.slot_dep.data(), nslot * 8);
+        memcpy(&host[w.ori], T.rinfo.data(), T.rinfo.size() * 4);
+        memcpy(&host[w.oli], T.list.data(), T.list.size() * 4);
+        memcpy(&host[w.ost], T.step.data(), T.step.size() * 4);
+        cudaError_t e = dev_malloc((void **)&w.buf, w.bytes);
+        if (e == cudaSuccess) e = cudaMemcpy(w.buf, host.data(), w.ovar, cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) return cuda_status(e, "window lists");
+    }
+    return XD_OK;
+}
+
+// The lists of win_ham_lists, and the coefficients and diagonals of every pass
+// for the handle's couplings.
+xd_status win_ham_tables(xd_ham_s *h, std::vector<WinPassHam> *lists) {
     const xd_basis_s *b = h->b;
     const WinLayoutHost &wl = b->win;
     const int np = (int)wl.pairs.size();
+    h->win.resize(wl.pass.size());
+    // products in flight on any stream read the lists that go
+    bool replaced = false;
+    for (size_t ip = 0; ip < lists->size(); ++ip) replaced = replaced || (h->win[ip].buf && (*lists)[ip].buf);
+    if (replaced) XD_CUDA(cudaDeviceSynchronize());
+    std::fill(h->win_fit, h->win_fit + kWinForms, true);
+    for (size_t ip = 0; ip < lists->size(); ++ip) {
+        WinPassHam &w = h->win[ip];
+        if ((*lists)[ip].buf) {
+            cudaFree(w.buf);
+            w = (*lists)[ip];
+            (*lists)[ip].buf = nullptr;
+        }
+        for (int f = 0; f < kWinForms; ++f) h->win_fit[f] = h->win_fit[f] && w.fit[f];
+    }
     double q = 1.0;
     std::vector<int> k;
     h->x64_fx_ok = find_quantum(h->J, &q, &k);
-    std::vector<double> Jp(np, 0.0);
+    const std::vector<double> Jp = pair_couplings(b, h->J.data());
     std::vector<int> kp(np, 0);
     int64_t kabs = 0;
-    for (int t = 0; t < b->nb; ++t) {
-        Jp[wl.pair_of[t]] += h->J[t];
-        if (h->x64_fx_ok) {
-            kp[wl.pair_of[t]] += k[t];
-            kabs += std::abs(k[t]);
-        }
+    for (int t = 0; t < b->nb && h->x64_fx_ok; ++t) {
+        kp[wl.pair_of[t]] += k[t];
+        kabs += std::abs(k[t]);
     }
     // every partial sum is at most 3 sum|k_b| max|X| < 2^62
     int lg = 0;
     while ((int64_t(1) << lg) < 3 * std::max<int64_t>(1, kabs)) ++lg;
     h->x64_B = 62 - lg;
     h->x64_qs = 0.25 * q;
-    const bool wide = win_wide(b->dim_u1);
-    h->win.resize(wl.pass.size());
-    std::fill(h->win_fit, h->win_fit + kWinForms, true);
     for (size_t ip = 0; ip < wl.pass.size(); ++ip) {
-        const WinPassDev &pd = wl.pass[ip];
-        WinPassHam &w = h->win[ip];
-        const WinPass &p = pd.p;
+        const WinPassHam &w = h->win[ip];
+        const WinPass &p = wl.pass[ip].p;
         const int nwb = (int)p.bonds.size(), ws = (int)p.S.size();
-        std::vector<double> vals;
-        std::vector<int> gid(nwb);
-        for (int t = 0; t < nwb; ++t) {
-            const double v = Jp[p.bonds[t]];
-            gid[t] = (int)(std::find(vals.begin(), vals.end(), v) - vals.begin());
-            if (gid[t] == (int)vals.size()) vals.push_back(v);
-        }
-        const int groups = (int)vals.size() <= kWinMaxGroups ? (int)vals.size() : 0;
-        if (!groups) gid.assign(nwb, 0);
-        const bool fresh = !w.buf || w.groups != groups || w.gid != gid;
-        auto up16 = [](size_t v) { return (v + 15) / 16 * 16; };
-        if (fresh) {
-            WinTables T;
-            w.ng = win_fitting_lists(p, wl.pairs, pd.nbase, wide, gid, groups, &T, w.fit);
-            w.ncoef = w.ng ? w.ng : kWinMaxBonds + 1;
-            w.groups = groups;
-            w.gid = gid;
-            w.slot_word = T.slot_word;
-            w.maxslots = T.maxslots;
-            w.maxlist = T.maxlist;
-            w.maxstep = T.maxstep;
-            const size_t nslot = T.slot_word.size();
-            size_t o = 0;
-            auto take = [&](size_t bytes) {
-                const size_t at = o;
-                o += up16(bytes);
-                return at;
-            };
-            const size_t oks = take(T.k.size() * sizeof(WinK)), osd = take(nslot * 8), ori = take(T.rinfo.size() * 4),
-                         oli = take(T.list.size() * 4), ost = take(T.step.size() * 4);
-            const size_t ovar = o;
-            size_t oc[3], od[3];
-            const size_t cs[3] = {8, 4, 4};
-            for (int a = 0; a < 3; ++a) {
-                oc[a] = take((kWinMaxBonds + 1) * cs[a]);
-                od[a] = take(nslot * cs[a]);
-            }
-            if (w.cap < o) {
-                cudaFree(w.buf);
-                w.buf = nullptr;
-                w.cap = 0;
-                XD_CUDA(dev_malloc((void **)&w.buf, o));
-                w.cap = o;
-            }
-            std::vector<unsigned char> host(ovar, 0);
-            memcpy(&host[oks], T.k.data(), T.k.size() * sizeof(WinK));
-            memcpy(&host[osd], T.slot_dep.data(), nslot * 8);
-            memcpy(&host[ori], T.rinfo.data(), T.rinfo.size() * 4);
-            memcpy(&host[oli], T.list.data(), T.list.size() * 4);
-            memcpy(&host[ost], T.step.data(), T.step.size() * 4);
-            XD_CUDA(cudaMemcpy(w.buf, host.data(), ovar, cudaMemcpyHostToDevice));
-            w.oks = oks;
-            w.osd = osd;
-            w.ori = ori;
-            w.oli = oli;
-            w.ost = ost;
-            w.ovar = ovar;
-            w.bytes = o;
-            for (int a = 0; a < 3; ++a) {
-                w.oc[a] = oc[a];
-                w.od[a] = od[a];
-            }
-        }
         // coefficients (double-float, fixed point, FP32) and the window words' diagonals
         auto pair = [](double d) {
             const float c = (float)d;
@@ -1049,7 +1064,7 @@ xd_status win_ham_tables(xd_ham_s *h) {
         std::vector<int> Dk(1u << ws, 0);
         for (int t = 0; t < nwb; ++t) {
             const auto &pr = wl.pairs[p.bonds[t]];
-            const int at = w.ng ? gid[t] : t, kb = kp[p.bonds[t]];
+            const int at = w.ng ? w.gid[t] : t, kb = kp[p.bonds[t]];
             const double j = Jp[p.bonds[t]];
             c0[at] = pair(0.5 * j);
             c1[at] = 2 * kb;
@@ -1073,7 +1088,6 @@ xd_status win_ham_tables(xd_ham_s *h) {
             d2[s] = (float)Dj[v];
         }
         XD_CUDA(cudaMemcpy(w.buf + w.ovar, var.data(), var.size(), cudaMemcpyHostToDevice));
-        for (int f = 0; f < kWinForms; ++f) h->win_fit[f] = h->win_fit[f] && w.fit[f];
     }
     return XD_OK;
 }
