@@ -72,7 +72,10 @@ namespace {
 
 // ------------------------------------------------------------- arithmetics
 // V: staged values; Acc: partial sums (as large as V); C: flip coefficient;
-// D: diagonal of a window word; Y: result.
+// D: diagonal of a window word; Y: result.  Lists coupling by coupling: list adds
+// a value of a coupling's part, mul_add that part's sum with its coefficient; in
+// FP32 list multiplies (an FMA costs what an addition does), because a sum of x
+// alone can overflow where no J x and no sum of them does.
 struct PolDF {
     static constexpr int kArith = 0;
     using V = float2;     // scaled x as (hi, lo)
@@ -91,7 +94,8 @@ struct PolDF {
         a.s = r.x;
         a.c = r.y;
     }
-    __device__ static void add(Acc &a, V v, V w) {
+    __device__ static void list(Acc &a, C, V v) { add(a, v); }
+    __device__ static void list(Acc &a, C, V v, V w) {
         add(a, v);
         add(a, w);
     }
@@ -117,8 +121,8 @@ struct PolFX {
         bool nan;
     };
     __device__ static void zero(Acc &a) { a.a = 0; }
-    __device__ static void add(Acc &a, V v) { a.a += v; }
-    __device__ static void add(Acc &a, V v, V w) { a.a = a.a + v + w; }  // three-input adds
+    __device__ static void list(Acc &a, C, V v) { a.a += v; }
+    __device__ static void list(Acc &a, C, V v, V w) { a.a = a.a + v + w; }  // three-input adds
     __device__ static void mul_add(Acc &a, C c, Acc s) { a.a += (long long)c * s.a; }
     __device__ static void fma(Acc &a, C c, V v) { a.a += (long long)c * v; }
     __device__ static void diag(Acc &a, D d, V v) { a.a += (long long)d * v; }
@@ -143,9 +147,9 @@ struct PolF32 {
     };
     struct Out {};
     __device__ static void zero(Acc &a) { a.a = 0.f; }
-    __device__ static void add(Acc &a, V v) { a.a += v; }
-    __device__ static void add(Acc &a, V v, V w) { a.a = (a.a + v) + w; }
-    __device__ static void mul_add(Acc &a, C c, Acc s) { a.a = fmaf(c, s.a, a.a); }
+    __device__ static void list(Acc &a, C c, V v) { a.a = fmaf(c, v, a.a); }
+    __device__ static void list(Acc &a, C c, V v, V w) { a.a = fmaf(c, w, fmaf(c, v, a.a)); }
+    __device__ static void mul_add(Acc &a, C, Acc s) { a.a += s.a; }
     __device__ static void fma(Acc &a, C c, V v) { a.a = fmaf(c, v, a.a); }
     __device__ static void diag(Acc &a, D d, V v) { a.a = fmaf(d, v, a.a); }
     __device__ static void merge(Acc &a, Acc b) { a.a += b.a; }
@@ -337,6 +341,7 @@ __device__ __forceinline__ void row_flips(const unsigned char *tile, const uint2
 #pragma unroll 1
         for (int g = 0; g < ng; ++g, counts >>= 8) {
             const int n = (int)(counts & 255u);
+            const typename Pol::C c = coef[g];
             Acc s[2][VL];
 #pragma unroll
             for (int i = 0; i < VL; ++i) {
@@ -352,9 +357,9 @@ __device__ __forceinline__ void row_flips(const unsigned char *tile, const uint2
                 q1.q = *(const int4 *)(tile + (e >> 16));
                 q3.q = *(const int4 *)(tile + (f >> 16));
 #pragma unroll
-                for (int k = 0; k < VL; ++k) Pol::add(s[0][k], q0.v[k], q1.v[k]);
+                for (int k = 0; k < VL; ++k) Pol::list(s[0][k], c, q0.v[k], q1.v[k]);
 #pragma unroll
-                for (int k = 0; k < VL; ++k) Pol::add(s[1][k], q2.v[k], q3.v[k]);
+                for (int k = 0; k < VL; ++k) Pol::list(s[1][k], c, q2.v[k], q3.v[k]);
             };
 #pragma unroll 1
             for (int i = n >> 2; i > 0; --i, lp += kWinRows) {
@@ -375,12 +380,11 @@ __device__ __forceinline__ void row_flips(const unsigned char *tile, const uint2
                     q0.q = *(const int4 *)(tile + ((e.x ^ c16) & 0xffffu));
                     q1.q = *(const int4 *)(tile + ((f.x ^ c16) & 0xffffu));
 #pragma unroll
-                    for (int k = 0; k < VL; ++k) Pol::add(s[0][k], q0.v[k]);
+                    for (int k = 0; k < VL; ++k) Pol::list(s[0][k], c, q0.v[k]);
 #pragma unroll
-                    for (int k = 0; k < VL; ++k) Pol::add(s[1][k], q1.v[k]);
+                    for (int k = 0; k < VL; ++k) Pol::list(s[1][k], c, q1.v[k]);
                 }
             }
-            const typename Pol::C c = coef[g];
 #pragma unroll
             for (int k = 0; k < VL; ++k) {
                 Pol::mul_add(a[0][k], c, s[0][k]);
