@@ -355,7 +355,7 @@ xd_status build_big(Plan *p) {
     }
     p->ubig = units;
     p->smem8 = smem;
-    XD_CUDA(cudaFuncSetAttribute(k_batch8, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    XD_CUDA(allow_smem(k_batch8));
     XD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p->per_sm8, k_batch8, sp8::kT8, smem));
     if (p->per_sm8 < 1) {
         set_error("batched product: %zu bytes of shared memory do not fit", smem);

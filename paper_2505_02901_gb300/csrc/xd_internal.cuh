@@ -33,6 +33,19 @@ constexpr int kMaxBonds = 4096;
 // cudaMalloc, unless an allocation failure was injected (xd_debug_fail_alloc):
 // every device allocation of the library goes through here.
 cudaError_t dev_malloc(void **p, size_t bytes);
+
+// Lets a kernel's launches have all the shared memory of a CTA beside the
+// kernel's own: the limit and not a launch's size, because another thread may be
+// about to launch a larger one.
+constexpr int kCtaSmem = 227 * 1024;
+template <typename F>
+cudaError_t allow_smem(F *kern) {
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, (const void *)kern);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kCtaSmem - (int)a.sharedSizeBytes);
+}
+
 constexpr int kMaxGroup = 2048;
 constexpr int kMaxN = 40;
 

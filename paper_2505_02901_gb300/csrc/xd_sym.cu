@@ -889,11 +889,11 @@ xd_status sym_apply(const xd_ham_s *h, const void *x, void *y, xd_dtype dt, cuda
     };
     if (dt == XD_C128) {
         auto kern = pick(std::true_type());
-        XD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        XD_CUDA(allow_smem(kern));
         kern<<<grid, kThreads, smem, st>>>(v, sbo, nb, jq, b->d_chi, w.sq, (const double2 *)x, (double2 *)y);
     } else {
         auto kern = pick(std::false_type());
-        XD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        XD_CUDA(allow_smem(kern));
         kern<<<grid, kThreads, smem, st>>>(v, sbo, nb, jq, b->d_chi, w.sq, (const double *)x, (double *)y);
     }
     XD_CUDA(cudaGetLastError());

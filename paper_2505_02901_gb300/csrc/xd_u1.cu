@@ -212,7 +212,7 @@ static xd_status launch_apply(const xd_ham_s *h, const void *x, void *y, cudaStr
     const int nb = h->b->nb;
     size_t smem = (size_t)nb * (sizeof(uint64_t) + sizeof(T)) + (kFixRow<T> && nb <= kFixBonds ? (nb + 1) * sizeof(long long) : 0);
     auto kern = kVecRow<T, NV> && (((uintptr_t)x | (uintptr_t)y) & 15) == 0 ? k_apply<T, NV, kVecRow<T, NV>> : k_apply<T, NV, false>;
-    if (smem > 48 * 1024) XD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 48 * 1024) XD_CUDA(allow_smem(kern));
     int grid = grid_for(u.dim, kThreads, 8);
     kern<<<grid, kThreads, smem, st>>>(u, bondbuf, nb, (const T *)x, (T *)y);
     XD_CUDA(cudaGetLastError());

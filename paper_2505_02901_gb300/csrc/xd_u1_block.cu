@@ -411,7 +411,7 @@ static xd_status launch_block(const xd_ham_s *h, const void *x, void *y, cudaStr
     p.maxblk = Geo<L>::maxblk;
     const SmemLayout<T> lay(p, NBUF);
     auto kern = k_block_apply<T, L, NBUF>;
-    XD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.total));
+    XD_CUDA(allow_smem(kern));
     int per_sm = 0;
     XD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kBT, lay.total));
     if (per_sm < 1) {

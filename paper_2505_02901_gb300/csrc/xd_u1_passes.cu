@@ -807,7 +807,7 @@ static xd_status launch_passes(const xd_ham_s *h, const typename Pol::V *x, type
         const size_t tsm = TPassSmem(tp.ws, tp.nwb, sizeof(typename Pol::V), sizeof(typename Pol::C),
                                      sizeof(typename Pol::Acc), q == 0).total;
         auto tk = q == 0 ? k_tpass<Pol, true> : k_tpass<Pol, false>;
-        XD_CUDA(cudaFuncSetAttribute(tk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm));
+        XD_CUDA(allow_smem(tk));
         int tper = 0;
         XD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&tper, tk, kT, tsm));
         if (tper < 1) {
@@ -846,7 +846,7 @@ static xd_status launch_passes(const xd_ham_s *h, const typename Pol::V *x, type
     p.state = h->d_x64_state;
     const MainSmem<Pol, KB> lay(p);
     auto kern = k_main<Pol, KB>;
-    XD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.total));
+    XD_CUDA(allow_smem(kern));
     int per_sm = 0;
     XD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kT, lay.total));
     if (per_sm < 1) {

@@ -580,7 +580,7 @@ static xd_status launch_spmm(const xd_ham_s *h, const void *x, void *y, cudaStre
     p.jcross = h->sp_jcross;
     const SpSmem lay(p, SpGeo<L>::maxblk);
     auto kern = k_spmm<L>;
-    XD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.total));
+    XD_CUDA(allow_smem(kern));
     int per_sm = 0;
     XD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kT, lay.total));
     if (per_sm < 1) {

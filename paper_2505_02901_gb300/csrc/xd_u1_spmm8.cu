@@ -44,7 +44,7 @@ xd_status launch_spmm8(const xd_ham_s *h, const float *x, float *y, cudaStream_t
     sp8_params(h, &p);
     const Sp8Smem lay(p, Sp8Geo<L>::maxblk);
     auto kern = k_spmm8<L>;
-    XD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.total));
+    XD_CUDA(allow_smem(kern));
     int per_sm = 0;
     XD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kT8, lay.total));
     if (per_sm < 1) {
