@@ -121,13 +121,9 @@ inline std::vector<WinPass> choose_windows(int N, int nup, const std::vector<std
         full[p.first] |= 1ull << p.second;
         full[p.second] |= 1ull << p.first;
     }
-    auto inside = [&](const Adj &a, uint64_t S) {  // uncovered pairs inside S
-        int c = 0;
-        for (uint64_t t = S; t; t &= t - 1) c += pop(a[__builtin_ctzll(t)] & S);
-        return c / 2;
-    };
     std::vector<uint64_t> best;
     double best_cost = 0;
+    int deg[64], near[64];
     // no window covers more pairs than the best one does at the start
     int most = 1;
     for (int trial = 0, quiet = 0; trial < 96 && quiet < 24; ++trial, ++quiet) {
@@ -142,13 +138,31 @@ inline std::vector<WinPass> choose_windows(int N, int nup, const std::vector<std
         std::vector<uint64_t> wins;
         int left = n;
         while (left > 0 && (best.empty() || wins.size() < best.size())) {  // as many windows as the best, or fewer
+            uint64_t open = 0;  // sites of uncovered pairs
+            int low_pairs = 0, nopen = 0;
+            for (int v = 0; v < N; ++v) {
+                deg[v] = pop(a[v]);
+                open |= (uint64_t)(a[v] != 0) << v;
+                nopen += a[v] != 0;
+                if (v < kWinLow) low_pairs += pop(a[v] & low);
+            }
             int bc = 0, b1 = -(1 << 30), b2 = 0;
             uint32_t bl = 0;
             uint64_t bs = 0;
+            // near: per site its uncovered pairs with S, kept as S grows
+            auto grow = [&](uint64_t u) {
+                for (uint64_t t = u & open; t; t &= t - 1)
+                    for (uint64_t q = a[__builtin_ctzll(t)]; q; q &= q - 1) ++near[__builtin_ctzll(q)];
+            };
             auto consider = [&](uint64_t S) {
-                int cnt = inside(a, S), r = 0;
+                int cnt = 0, r = nopen;  // uncovered pairs inside S, sites that the others touch
+                for (uint64_t t = S & open; t; t &= t - 1) {
+                    const int v = __builtin_ctzll(t);
+                    cnt += near[v];
+                    r -= near[v] == deg[v];
+                }
+                cnt /= 2;
                 if (cnt == 0) return;
-                for (int v = 0; v < N; ++v) r += (a[v] & ~(((S >> v) & 1) ? S : 0ull)) != 0;
                 bool rows = false;
                 const uint32_t tie = trial == 0 ? (uint32_t)std::min(runs(S, &rows), 8) : next() & 0xffffu;
                 const bool sites = trial & 1;  // odd trials: the fewest sites left first
@@ -164,32 +178,42 @@ inline std::vector<WinPass> choose_windows(int N, int nup, const std::vector<std
             for (int v0 = 0; v0 < N; ++v0) {
                 uint64_t S = unit(v0);
                 for (int v = (v0 + 1) % N; pop(S | unit(v)) <= W && v != v0; v = (v + 1) % N) S |= unit(v);
+                std::fill(near, near + N, 0);
+                grow(S);
                 consider(S);
             }
             for (int start = 0; start < N; ++start) {
                 if (!a[start]) continue;
-                uint64_t S = unit(start);
-                for (;;) {
-                    uint64_t bu = 0;
+                uint64_t S = 0;
+                int size = 0;
+                std::fill(near, near + N, 0);
+                for (uint64_t bu = unit(start); bu;) {
+                    S |= bu;
+                    size += bu == low ? kWinLow : 1;
+                    grow(bu);
+                    bu = 0;
                     int bg = 0;
-                    for (int v = 0; v < N; ++v) {
-                        const uint64_t u = unit(v);
-                        if ((S & u) || (v > 0 && v < kWinLow) || pop(S | u) > W) continue;
-                        int g = 0, d = 0;
-                        for (uint64_t t = u; t; t &= t - 1) {
-                            const uint64_t nb = a[__builtin_ctzll(t)];
-                            g += 2 * pop(nb & S) + pop(nb & u);
-                            d += pop(nb);
-                        }
+                    auto offer = [&](uint64_t u, int g, int d) {
                         // pairs gained first, then the remaining degree (trial 0) or chance
                         const int score = g * 4096 + (trial == 0 ? d * 16 : (int)(next() & 1023u)) + 1;
                         if (g > 0 && score > bg) {
                             bg = score;
                             bu = u;
                         }
+                    };
+                    if (!(S & low) && size + kWinLow <= W) {
+                        int g = low_pairs, d = 0;
+                        for (int v = 0; v < std::min(N, kWinLow); ++v) {
+                            g += 2 * near[v];
+                            d += deg[v];
+                        }
+                        offer(low, g, d);
                     }
-                    if (!bu) break;
-                    S |= bu;
+                    if (size < W)
+                        for (uint64_t t = ~S & all & ~low; t; t &= t - 1) {
+                            const int v = __builtin_ctzll(t);
+                            offer(1ull << v, 2 * near[v], deg[v]);
+                        }
                 }
                 consider(S);
             }
@@ -214,6 +238,7 @@ inline std::vector<WinPass> choose_windows(int N, int nup, const std::vector<std
         }
         // while fewer windows may do, go on; then a few more for better runs
         if ((int)best.size() > (n + most - 1) / most || best.size() < before) quiet = 0;
+        else if (best_cost < (double)best.size() + 0.03) break;  // no window fewer, and little better runs
     }
     std::vector<WinPass> out;
     std::vector<char> cov(n, 0);
@@ -546,8 +571,19 @@ inline void win_lists(const WinPass &p, const std::vector<std::pair<int, int>> &
     win_shape(p, cl, T);
     const int ws = (int)p.S.size(), nwb = (int)p.bonds.size(), nsub = 2 * std::max(1, ng);
     const std::vector<uint32_t> &masks = cl.masks;
-    int sub[kWinMaxBonds + 1];  // group and whether the flip changes the parity
-    for (int b = 0; b < nwb; ++b) sub[b] = 2 * (ng ? gid[b] : 0) + (__builtin_popcount(cl.colour & masks[b]) == 1 ? 0 : 1);
+    uint64_t sub[2 * kWinMaxGroups] = {};  // the bonds of a group whose flips change the parity, and keep it
+    uint64_t at_site[kWinSites] = {};
+    for (int b = 0; b < nwb; ++b) {
+        sub[2 * (ng ? gid[b] : 0) + (__builtin_popcount(cl.colour & masks[b]) == 1 ? 0 : 1)] |= 1ull << b;
+        for (uint32_t t = masks[b]; t; t &= t - 1) at_site[__builtin_ctz(t)] |= 1ull << b;
+    }
+    // a word's flipping bonds have one site up: the XOR of the bonds at its up sites
+    std::vector<uint64_t> flips(1u << ws, 0), dep(1u << ws, 0);
+    for (uint32_t w = 1; w < (1u << ws); ++w) {
+        const int v = __builtin_ctz(w);
+        flips[w] = flips[w & (w - 1)] ^ at_site[v];
+        dep[w] = dep[w & (w - 1)] | 1ull << p.S[v];
+    }
     const size_t nslots = T->k[ws].slot0 + kWinRows * T->k[ws].nstep;
     T->slot_word.assign(nslots, 0xffffu);
     T->slot_dep.assign(nslots, ~0ull);
@@ -556,18 +592,17 @@ inline void win_lists(const WinPass &p, const std::vector<std::pair<int, int>> &
     T->maxlist = 0;
     T->rinfo.assign(1u << ws, 0);
     std::vector<uint16_t> slot_of(1u << ws, 0);
-    std::vector<std::pair<uint64_t, uint32_t>> cls[2];
-    uint16_t ent[kWinRows][2 * kWinMaxGroups][kWinMaxBonds];
+    std::vector<uint64_t> cls[2];  // per parity: the numbers of flips (six bits each), then the word
+    constexpr uint64_t kWord = (1ull << kWinSites) - 1;
+    static_assert(6 * 2 * kWinMaxGroups + kWinSites <= 64 && kWinMaxBonds < 64, "counts and word in 64 bits");
     for (int k = 0; k <= ws; ++k) {
         WinK &K = T->k[k];
         const std::vector<uint32_t> &words = cl.words[k];
         for (auto &c : cls) c.clear();
         for (uint32_t w : words) {
-            int cnt[2 * kWinMaxGroups] = {};
-            for (int b = 0; b < nwb; ++b) cnt[sub[b]] += (w & masks[b]) != 0 && (w & masks[b]) != masks[b];
             uint64_t key = 0;
-            for (int s = 0; s < nsub; ++s) key = key << 7 | (uint64_t)cnt[s];
-            cls[__builtin_popcount(w & cl.colour) & 1].push_back({key, w});
+            for (int s = 0; s < nsub; ++s) key = key << 6 | (uint64_t)__builtin_popcountll(flips[w] & sub[s]);
+            cls[__builtin_popcount(w & cl.colour) & 1].push_back(key << kWinSites | w);
         }
         for (auto &c : cls) std::sort(c.begin(), c.end());
         K.step0 = (int)T->step.size() / 2;
@@ -575,24 +610,18 @@ inline void win_lists(const WinPass &p, const std::vector<std::pair<int, int>> &
         for (int c = 0; c < 2; ++c)
             for (size_t i = 0; i < cls[c].size(); ++i) {
                 const int slot = 2 * (int)i + c;
-                T->slot_word[K.slot0 + slot] = (uint16_t)cls[c][i].second;
-                T->slot_dep[K.slot0 + slot] = win_deposit(cls[c][i].second, p.S);
-                slot_of[cls[c][i].second] = (uint16_t)slot;
+                const uint32_t w = (uint32_t)(cls[c][i] & kWord);
+                T->slot_word[K.slot0 + slot] = (uint16_t)w;
+                T->slot_dep[K.slot0 + slot] = dep[w];
+                slot_of[w] = (uint16_t)slot;
             }
         uint32_t pos = 0;  // fours of entries written for this k
         for (int o = 0; o < K.nstep; ++o) {
-            int n[kWinRows][2 * kWinMaxGroups] = {}, mx[2 * kWinMaxGroups] = {};
-            for (int r = 0; r < kWinRows; ++r) {
-                const uint32_t w = T->slot_word[K.slot0 + kWinRows * o + r];
-                if (w == 0xffffu) continue;
-                for (int b = 0; b < nwb; ++b) {
-                    const uint32_t t = w & masks[b];
-                    if (t == 0 || t == masks[b]) continue;
-                    const uint32_t s = slot_of[w ^ masks[b]];
-                    ent[r][sub[b]][n[r][sub[b]]++] = (uint16_t)(ng ? win_row_off(p.rows, s) : (s | (uint32_t)b << 10));
-                }
-                for (int s = 0; s < nsub; ++s) mx[s] = std::max(mx[s], n[r][s]);
-            }
+            const uint16_t *words_at = &T->slot_word[K.slot0 + kWinRows * o];
+            int mx[2 * kWinMaxGroups] = {};
+            for (int r = 0; r < kWinRows; ++r)
+                for (int s = 0; s < nsub && words_at[r] != 0xffffu; ++s)
+                    mx[s] = std::max(mx[s], __builtin_popcountll(flips[words_at[r]] & sub[s]));
             T->step.push_back(pos);
             uint32_t counts = 0;
             for (int g = 0; g < nsub / 2; ++g) {
@@ -604,10 +633,21 @@ inline void win_lists(const WinPass &p, const std::vector<std::pair<int, int>> &
                     const uint32_t z0 = (uint32_t)(kWinRows * K.nstep) + ((r & 1) ^ 1), z1 = (uint32_t)(kWinRows * K.nstep) + (r & 1);
                     const uint32_t pad0 = ng ? win_row_off(p.rows, z0) : (z0 | (uint32_t)kWinMaxBonds << 10);
                     const uint32_t pad1 = ng ? win_row_off(p.rows, z1) : (z1 | (uint32_t)kWinMaxBonds << 10);
-                    for (int e = 0; e < m; ++e) {
-                        const int keep = e < mx[2 * g] ? 0 : 1, i = keep ? e - mx[2 * g] : e;
-                        const uint32_t v = i < n[r][2 * g + keep] ? ent[r][2 * g + keep][i] : keep ? pad1 : pad0;
-                        T->list[K.list0 + (size_t)(pos + e / 4) * 2 * kWinRows + 2 * r + ((e >> 1) & 1)] |= v << (16 * (e & 1));
+                    uint32_t *at = &T->list[K.list0 + (size_t)pos * 2 * kWinRows + 2 * r];
+                    const uint32_t w = words_at[r];
+                    int e = 0;
+                    for (int keep = 0; keep < 2; ++keep) {
+                        uint64_t t = w == 0xffffu ? 0 : flips[w] & sub[2 * g + keep];
+                        for (int i = 0; i < mx[2 * g + keep]; ++i, ++e) {
+                            uint32_t v = keep ? pad1 : pad0;
+                            if (t) {
+                                const int b = __builtin_ctzll(t);
+                                const uint32_t s = slot_of[w ^ masks[b]];
+                                v = ng ? win_row_off(p.rows, s) : (s | (uint32_t)b << 10);
+                                t &= t - 1;
+                            }
+                            at[e / 4 * 2 * kWinRows + ((e >> 1) & 1)] |= v << (16 * (e & 1));
+                        }
                     }
                 }
                 pos += (uint32_t)(m + 3) / 4;
