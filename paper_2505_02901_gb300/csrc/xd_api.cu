@@ -473,7 +473,7 @@ static xd_status set_J(xd_ham_s *h, const double *J) {
     batch_forget(h);  // captured launches hold per-coupling scalars and addresses
     h->J.assign(J, J + b->nb);
     XD_CUDA(cudaMemcpy(h->d_J, J, sizeof(double) * b->nb, cudaMemcpyHostToDevice));
-    std::vector<double> buf(3 * b->nb + 2);
+    std::vector<double> buf(3 * b->nb + 5);
     double q = 0.0;
     for (int k = 0; k < b->nb; ++k) {
         buf[k] = J[k];
@@ -493,6 +493,12 @@ static xd_status set_J(xd_ham_s *h, const double *J) {
         const long long f = fits ? llrint(ldexp(0.5 * J[k], 62 - ex)) : 0;
         memcpy(&buf[2 * b->nb + 2 + k], &f, sizeof f);
     }
+    // FP32: sum J/4 in units of 2^(ex - 30), that unit as two factors
+    const long long jq = fits ? llrint(ldexp(0.25 * q, 30 - ex)) : 0;
+    const int half = (ex - 30) / 2;
+    memcpy(&buf[3 * b->nb + 2], &jq, sizeof jq);
+    buf[3 * b->nb + 3] = fits ? ldexp(1.0, half) : 0.0;
+    buf[3 * b->nb + 4] = fits ? ldexp(1.0, ex - 30 - half) : 0.0;
     XD_CUDA(cudaMemcpy(h->d_bond, buf.data(), sizeof(double) * buf.size(), cudaMemcpyHostToDevice));
     if (b->blk.ok) XD_TRY(block_ham_tables(h));
     if (b->spmm.ok) XD_TRY(spmm_ham_tables(h));
@@ -510,7 +516,7 @@ xd_status xd_ham_create(xd_basis b, const double *J, xd_ham *out) {
     auto *h = new xd_ham_s();
     h->b = b;
     cudaError_t e = dev_malloc((void **)&h->d_J, sizeof(double) * b->nb);
-    if (e == cudaSuccess) e = dev_malloc((void **)&h->d_bond, sizeof(double) * (3 * b->nb + 2));
+    if (e == cudaSuccess) e = dev_malloc((void **)&h->d_bond, sizeof(double) * (3 * b->nb + 5));
     if (e == cudaSuccess) e = dev_malloc((void **)&h->d_scal, sizeof(double) * 64);
     if (e != cudaSuccess) {
         cudaFree(h->d_J);

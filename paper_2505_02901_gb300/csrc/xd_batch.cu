@@ -50,11 +50,12 @@ struct Inst {
 
 constexpr int kMaxBatchBonds = 512;
 
+using u1rows::BondCoef;
 using u1rows::find_block;
 
-// Rows [row0, row1) of instance I (bond table staged in sm_mask / sm_half).
+// Rows [row0, row1) of instance I (bond table staged in sm_mask / sm_coef).
 template <typename T, int NV, bool VEC>
-__device__ __forceinline__ void batch_rows_at(const Inst &I, const uint64_t *sm_mask, const T *sm_half,
+__device__ __forceinline__ void batch_rows_at(const Inst &I, const uint64_t *sm_mask, const BondCoef<T> *sm_coef,
                                            uint64_t *sh_range, int64_t row0, int64_t row1) {
     const U1View &u = I.u;
     if (threadIdx.x == 0) {
@@ -64,7 +65,7 @@ __device__ __forceinline__ void batch_rows_at(const Inst &I, const uint64_t *sm_
         sh_range[1] = find_block(u.hi_off, h0, nh - 1, row1 - 1);
     }
     __syncthreads();
-    const T jq = (T)I.bond[2 * I.nb];
+    const u1rows::RowDiag<T> diag(I.bond, I.nb);
     const T *__restrict__ x = (const T *)I.x;
     T *__restrict__ y = (T *)I.y;
     for (int64_t r = row0 + threadIdx.x; r < row1; r += blockDim.x) {
@@ -75,10 +76,9 @@ __device__ __forceinline__ void batch_rows_at(const Inst &I, const uint64_t *sm_
         T acc[NV];
 #pragma unroll
         for (int q = 0; q < NV; ++q) acc[q] = T(0);
-        T dsub = T(0);
+        T d;
         // in turn: walked bits spill in k_batch8, whose registers the prefix blocks take
-        u1rows::row_flips<T, NV, false, VEC, false>(u, s, sm_mask, sm_half, I.nb, x, acc, dsub);
-        const T d = jq - dsub;
+        u1rows::row_flips<T, NV, false, VEC, false>(u, s, sm_mask, sm_coef, I.nb, x, acc, diag, d);
         T xr[NV];
         u1rows::load_row<T, NV, false, VEC>(x, r, xr);
 #pragma unroll
@@ -89,22 +89,12 @@ __device__ __forceinline__ void batch_rows_at(const Inst &I, const uint64_t *sm_
 
 // in 16-byte pieces where the instance's vectors allow it
 template <typename T, int NV>
-__device__ __forceinline__ void batch_rows(const Inst &I, const uint64_t *sm_mask, const T *sm_half,
+__device__ __forceinline__ void batch_rows(const Inst &I, const uint64_t *sm_mask, const BondCoef<T> *sm_coef,
                                            uint64_t *sh_range, int64_t row0, int64_t row1) {
     if (u1rows::kVecRow<T, NV> && (((uintptr_t)I.x | (uintptr_t)I.y) & 15) == 0)
-        batch_rows_at<T, NV, u1rows::kVecRow<T, NV>>(I, sm_mask, sm_half, sh_range, row0, row1);
+        batch_rows_at<T, NV, u1rows::kVecRow<T, NV>>(I, sm_mask, sm_coef, sh_range, row0, row1);
     else
-        batch_rows_at<T, NV, false>(I, sm_mask, sm_half, sh_range, row0, row1);
-}
-
-// Stages the bond table of instance I.
-template <typename T>
-__device__ __forceinline__ void batch_stage(const Inst &I, uint64_t *sm_mask, T *sm_half) {
-    const uint64_t *masks = (const uint64_t *)(I.bond + I.nb);
-    for (int b = threadIdx.x; b < I.nb; b += blockDim.x) {
-        sm_mask[b] = masks[b];
-        sm_half[b] = (T)(0.5 * I.bond[b]);
-    }
+        batch_rows_at<T, NV, false>(I, sm_mask, sm_coef, sh_range, row0, row1);
 }
 
 // Instance of global tile t: the last with tile0 <= t.
@@ -120,7 +110,7 @@ __device__ __forceinline__ int batch_find(const Inst *__restrict__ inst, int nin
 template <typename T, int NV>
 __global__ void k_batch(const Inst *__restrict__ inst, int ninst, int64_t ntiles, int tile_rows) {
     __shared__ uint64_t sm_mask[kMaxBatchBonds];
-    __shared__ T sm_half[kMaxBatchBonds];
+    __shared__ BondCoef<T> sm_coef[kMaxBatchBonds];
     __shared__ int sh_k;
     __shared__ uint64_t sh_range[2];
     int cur = -1;
@@ -130,11 +120,11 @@ __global__ void k_batch(const Inst *__restrict__ inst, int ninst, int64_t ntiles
         const int k = sh_k;
         const Inst &I = inst[k];
         if (k != cur) {
-            batch_stage(I, sm_mask, sm_half);
+            u1rows::stage_bonds(I.bond, I.nb, sm_mask, sm_coef);
             cur = k;
         }
         const int64_t row0 = (t - I.tile0) * tile_rows;
-        batch_rows<T, NV>(I, sm_mask, sm_half, sh_range, row0, min(row0 + (int64_t)tile_rows, I.u.dim));
+        batch_rows<T, NV>(I, sm_mask, sm_coef, sh_range, row0, min(row0 + (int64_t)tile_rows, I.u.dim));
         __syncthreads();
     }
 }
@@ -169,7 +159,7 @@ __global__ void __launch_bounds__(sp8::kT8, 2) k_batch8(const __grid_constant__ 
     __shared__ int sh_k;
     __shared__ long long sh_t;
     __shared__ uint64_t sm_mask[kMaxBatchBonds];
-    __shared__ float sm_half[kMaxBatchBonds];
+    __shared__ BondCoef<float> sm_coef[kMaxBatchBonds];
     __shared__ uint64_t sh_range[2];
     int cur_big = -1, cur_small = -1;
     const int64_t total = a.ubig + a.ntiles;
@@ -211,11 +201,11 @@ __global__ void __launch_bounds__(sp8::kT8, 2) k_batch8(const __grid_constant__ 
             const int k = sh_k;
             const Inst &I = a.inst[k];
             if (k != cur_small) {
-                batch_stage(I, sm_mask, sm_half);
+                u1rows::stage_bonds(I.bond, I.nb, sm_mask, sm_coef);
                 cur_small = k;
             }
             const int64_t row0 = (tt - I.tile0) * a.tile_rows;
-            batch_rows<float, 8>(I, sm_mask, sm_half, sh_range, row0, min(row0 + (int64_t)a.tile_rows, I.u.dim));
+            batch_rows<float, 8>(I, sm_mask, sm_coef, sh_range, row0, min(row0 + (int64_t)a.tile_rows, I.u.dim));
         }
         __syncthreads();  // unit done: shared state may be overwritten
     }

@@ -98,7 +98,7 @@ struct AccOf<float> {
 constexpr int kLzTabRow = 24, kLzTabBonds = 256, kLzTabBytes = 128 * 1024;
 template <typename T>
 __host__ __device__ inline size_t lz_tab_at(int nb) {
-    return ((size_t)nb * (sizeof(uint64_t) + sizeof(T)) + 15) / 16 * 16;
+    return ((size_t)nb * (sizeof(uint64_t) + sizeof(u1rows::BondCoef<T>)) + 15) / 16 * 16;
 }
 
 // Vector updates with their roundings spelt out (a product, then one fused
@@ -298,33 +298,37 @@ struct LzRow {
     uint64_t s;
     bool valid;
     int n = 0;
-    T dsub = T(0);
+    const u1rows::RowDiag<T> diag;
+    T d = T(0);
     const uint64_t *mask;
-    const T *half;
+    const u1rows::BondCoef<T> *coef;
     uint32_t *tab;
     int nb;
 
     __device__ __forceinline__ LzRow(const U1View &u1, const double *bond, int nb_, unsigned char *smem, int64_t r,
-                                     uint64_t *sh_range) : nb(nb_) {
+                                     uint64_t *sh_range) : diag(bond, nb_), nb(nb_) {
         uint64_t *m = (uint64_t *)smem;
-        T *hf = (T *)(m + nb);
-        u1rows::stage_bonds(bond, nb, m, hf);
+        u1rows::BondCoef<T> *c = (u1rows::BondCoef<T> *)(m + nb);
+        u1rows::stage_bonds(bond, nb, m, c);
         mask = m;
-        half = hf;
+        coef = c;
         tab = (uint32_t *)(smem + lz_tab_at<T>(nb)) + threadIdx.x;
         const u1rows::RowState rs = u1rows::unrank_tile(u1, (int64_t)blockIdx.x * blockDim.x, r, sh_range);
         s = rs.s;
         valid = rs.valid;
-        if (TAB && valid)
+        if (TAB && valid) {
+            u1rows::DiagSum<T> dsub;
             for (int b = 0; b < nb; ++b) {
                 const uint64_t t = s & mask[b];
                 if (t == 0 || t == mask[b]) continue;
                 tab[kThreads * n++] = (uint32_t)u1rows::rank_of(u1, s ^ mask[b]) | (uint32_t)b << kLzTabRow;
-                dsub += half[b];
+                dsub.add(coef[b]);
             }
+            d = dsub.diagonal(diag);
+        }
     }
-    __device__ __forceinline__ T product(const U1View &u1, const T *u, T ur, T jq) const {
-        T acc[1] = {T(0)}, d = dsub;
+    __device__ __forceinline__ T product(const U1View &u1, const T *u, T ur) const {
+        T acc[1] = {T(0)}, dr = d;
         if (TAB) {
             constexpr int D = 8;
             for (int j = 0; j < n; j += D) {
@@ -338,12 +342,12 @@ struct LzRow {
                     }
 #pragma unroll
                 for (int q = 0; q < D; ++q)
-                    if (j + q < n) acc[0] = fma_rn(half[e[q] >> kLzTabRow], x[q], acc[0]);
+                    if (j + q < n) acc[0] = fma_rn(coef[e[q] >> kLzTabRow].h, x[q], acc[0]);
             }
         } else {
-            u1rows::row_flips<T, 1, true, false>(u1, s, mask, half, nb, u, acc, d);
+            u1rows::row_flips<T, 1, true, false>(u1, s, mask, coef, nb, u, acc, diag, dr);
         }
-        return fma_rn(jq - d, ur, acc[0]);
+        return fma_rn(dr, ur, acc[0]);
     }
 };
 
@@ -369,7 +373,6 @@ __global__ void __launch_bounds__(kThreads) k_lz_persist(U1View u1, const double
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint64_t sh_range[2];
     __shared__ double sh_sum[2];
-    const T jq = (T)bond[2 * nb];
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // this thread's row
     const LzRow<T, TAB> row(u1, bond, nb, smem, r, sh_range);
     double sig = sd->sig, cz = sd->cz, amax = sd->amax;
@@ -381,7 +384,7 @@ __global__ void __launch_bounds__(kThreads) k_lz_persist(U1View u1, const double
         double d1 = 0.0, d2 = 0.0;
         if (row.valid) {
             const T ur = u[r];
-            const T wr = row.product(u1, u, ur, jq);
+            const T wr = row.product(u1, u, ur);
             w[r] = wr;
             d1 = (double)wr * (double)ur;
             d2 = (double)up[r] * (double)ur;
@@ -446,7 +449,6 @@ __global__ void __launch_bounds__(kThreads) k_lz_persist2(U1View u1, const doubl
     cooperative_groups::grid_group grid = cooperative_groups::this_grid();
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint64_t sh_range[2];
-    const T jq = (T)bond[2 * nb];
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const LzRow<T, TAB> row(u1, bond, nb, smem, r, sh_range);
     T *u = b0, *w = b1;
@@ -456,7 +458,7 @@ __global__ void __launch_bounds__(kThreads) k_lz_persist2(U1View u1, const doubl
         acc += (T)(abc[2 * steps + k] * sig) * ur;
         if (k == steps - 1) break;
         if (row.valid) {
-            const T wr = row.product(u1, u, ur, jq);
+            const T wr = row.product(u1, u, ur);
             const T t = fma_rn((T)(-abc[k] * sig), ur, fma_rn((T)cz, upr, mul_rn((T)sig, wr)));
             w[r] = t;
             upr = ur;

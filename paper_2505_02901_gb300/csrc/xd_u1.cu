@@ -23,21 +23,23 @@ constexpr int kThreads = 256;
 
 using namespace u1rows;
 
-// y = H x (the row loop of xd_u1_rows.cuh).
+// y = H x (the row loop of xd_u1_rows.cuh).  Eight FP32 columns in 48 registers,
+// five CTAs to an SM (us, in 60: 20 sites with 100 bonds 80 and 97, 21 sites 134 and
+// 144, 23 sites 506 and 445).
 template <typename T, int NV, bool VEC>
-__global__ void __launch_bounds__(kThreads) k_apply(U1View u, const double *__restrict__ bond,
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && NV == 8 ? 5 : 0) k_apply(U1View u, const double *__restrict__ bond,
                                                     int nb, const T *__restrict__ x,
                                                     T *__restrict__ y) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t *sm_mask = (uint64_t *)smem;
-    T *sm_half = (T *)(sm_mask + nb);
+    BondCoef<T> *sm_coef = (BondCoef<T> *)(sm_mask + nb);
     __shared__ uint64_t sh_range[2];
     const bool fixed = kFixRow<T> && nb <= kFixBonds && bond[2 * nb + 1] != 0.0;
-    long long *sm_fix = fixed ? (long long *)(sm_half + nb) : nullptr;
-    stage_bonds(bond, nb, sm_mask, sm_half, sm_fix);
-    const T jq = (T)bond[2 * nb];
+    long long *sm_fix = fixed ? (long long *)(sm_coef + nb) : nullptr;
+    stage_bonds(bond, nb, sm_mask, sm_coef, sm_fix);
+    const RowDiag<T> diag(bond, nb);
     __syncthreads();
-    apply_rows<T, NV, false, VEC>(u, sm_mask, sm_half, nb, jq, x, y, sh_range, sm_fix);
+    apply_rows<T, NV, false, VEC>(u, sm_mask, sm_coef, nb, diag, x, y, sh_range, sm_fix);
 }
 
 // State words of rows [first, first + count): the block of row r is the last
@@ -210,7 +212,7 @@ static xd_status launch_apply(const xd_ham_s *h, const void *x, void *y, cudaStr
     const double *bondbuf = h->d_bond;
     const U1View u = h->b->u1view();
     const int nb = h->b->nb;
-    size_t smem = (size_t)nb * (sizeof(uint64_t) + sizeof(T)) + (kFixRow<T> && nb <= kFixBonds ? (nb + 1) * sizeof(long long) : 0);
+    size_t smem = (size_t)nb * (sizeof(uint64_t) + sizeof(BondCoef<T>)) + (kFixRow<T> && nb <= kFixBonds ? (nb + 1) * sizeof(long long) : 0);
     auto kern = kVecRow<T, NV> && (((uintptr_t)x | (uintptr_t)y) & 15) == 0 ? k_apply<T, NV, kVecRow<T, NV>> : k_apply<T, NV, false>;
     if (smem > 48 * 1024) XD_CUDA(allow_smem(kern));
     int grid = grid_for(u.dim, kThreads, 8);

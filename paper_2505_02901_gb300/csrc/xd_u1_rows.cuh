@@ -123,14 +123,55 @@ __device__ __forceinline__ void store_row(T *y, int64_t r, const T (&v)[NV]) {
     }
 }
 
+// A bond's J/2; FP32 also has it in units of 2^-30 of a power of two above sum
+// |J/2|, for the diagonal.
+template <typename T>
+struct BondCoef {
+    T h;
+};
+template <>
+struct __align__(8) BondCoef<float> {
+    float h;
+    int f;
+};
+
+// The diagonal of a row, sum J/4 - sum over its flipping bonds of J/2.  The two
+// sums cancel to a few J, so FP32 takes them in the integers above: an integer
+// addition costs what an FP32 one does, and the error against 64 bits of a product
+// with random couplings falls (23 sites, 103 bonds 5.2e-7 with FP32 sums).
+template <typename T>
+struct RowDiag {
+    T jq;
+    __device__ __forceinline__ RowDiag(const double *__restrict__ bond, int nb) : jq(bond[2 * nb]) {}
+};
+template <>
+struct RowDiag<float> {
+    int jq;
+    float u1, u2;  // the unit in two factors, both normal numbers
+    __device__ __forceinline__ RowDiag(const double *__restrict__ bond, int nb)
+        : jq((int)*(const long long *)(bond + 3 * nb + 2)), u1((float)bond[3 * nb + 3]), u2((float)bond[3 * nb + 4]) {}
+};
+template <typename T>
+struct DiagSum {
+    T s = T(0);
+    __device__ __forceinline__ void add(BondCoef<T> c) { s += c.h; }
+    __device__ __forceinline__ T diagonal(const RowDiag<T> &g) const { return g.jq - s; }
+};
+template <>
+struct DiagSum<float> {
+    int s = 0;
+    __device__ __forceinline__ void add(BondCoef<float> c) { s += c.f; }
+    __device__ __forceinline__ float diagonal(const RowDiag<float> &g) const { return (float)(g.jq - s) * g.u1 * g.u2; }
+};
+
 // The flipping bonds of a row with state s, in ascending order: acc += J_b/2
-// x_c for each of the NV columns and dsub += J_b/2.  FP64 rows and rows of 32
+// x_c for each of the NV columns; d: the row's diagonal.  FP64 rows and rows of 32
 // bytes and more (WALK): the bonds are tested 32 at a time and then only the
 // set bits are walked, two targets being read together, so that a warp runs as
 // long as its row with the most flips and not once for every bond with half of
 // its lanes idle; the FP64 pipe, the limit in FP64, costs a warp the same
 // whether lanes are idle or not.  fix (or null; [nb], and then the unit): J_b/2
-// in integers, so that dsub costs that pipe one product a row and not one
+// in integers, so that the diagonal costs that pipe one product a row and not one
 // addition a flip.  FP64, in turn and now (us): 4x5 lattice, one column 55 and
 // 33, two 76 and 50; 22-site ladder, one 104 and 69; 4x6 lattice, two 1066 and
 // 706, eight 3058 and 2356 (2612 without the integers).  FP32, 22-site ladder,
@@ -143,20 +184,22 @@ template <typename T, int NV>
 constexpr bool kWalkRow = sizeof(T) == 8 || NV * sizeof(T) >= 32;
 
 template <typename T, int NV, bool COHERENT, bool VEC, bool WALK = kWalkRow<T, NV>>
-__device__ __forceinline__ void row_flips(const U1View &u, uint64_t s, const uint64_t *sm_mask, const T *sm_half, int nb,
-                                          const T *x, T (&acc)[NV], T &dsub, const long long *fix = nullptr) {
+__device__ __forceinline__ void row_flips(const U1View &u, uint64_t s, const uint64_t *sm_mask, const BondCoef<T> *sm_coef,
+                                          int nb, const T *x, T (&acc)[NV], const RowDiag<T> &diag, T &d,
+                                          const long long *fix = nullptr) {
     constexpr int D = 2;
     long long sum = 0;
+    DiagSum<T> dsub;
     if constexpr (!WALK) {
         for (int b = 0; b < nb; ++b) {
             const uint64_t mk = sm_mask[b], t = s & mk;
             if (t != 0 && t != mk) {
-                const T cf = sm_half[b];
+                const BondCoef<T> c = sm_coef[b];
                 T xv[NV];
                 load_row<T, NV, COHERENT, VEC>(x, rank_of(u, s ^ mk), xv);
 #pragma unroll
-                for (int k = 0; k < NV; ++k) acc[k] = fma_rn(cf, xv[k], acc[k]);
-                dsub += cf;
+                for (int k = 0; k < NV; ++k) acc[k] = fma_rn(c.h, xv[k], acc[k]);
+                dsub.add(c);
             }
         }
     } else {
@@ -176,7 +219,9 @@ __device__ __forceinline__ void row_flips(const U1View &u, uint64_t s, const uin
                     if (on[d]) {
                         const int b = b0 + __ffs(fl) - 1;
                         fl &= fl - 1;
-                        cf[d] = sm_half[b];
+                        const BondCoef<T> c = sm_coef[b];
+                        cf[d] = c.h;
+                        if constexpr (sizeof(T) == 4) dsub.add(c);
                         if (fix) sum += fix[b];
                         load_row<T, NV, COHERENT, VEC>(x, rank_of(u, s ^ sm_mask[b]), xv[d]);
                     }
@@ -186,12 +231,17 @@ __device__ __forceinline__ void row_flips(const U1View &u, uint64_t s, const uin
                     if (on[d]) {
 #pragma unroll
                         for (int k = 0; k < NV; ++k) acc[k] = fma_rn(cf[d], xv[d][k], acc[k]);
-                        if (!fix) dsub += cf[d];
+                        if constexpr (sizeof(T) == 8) {
+                            if (!fix) dsub.s += cf[d];
+                        }
                     }
             }
         }
     }
-    if (WALK && fix) dsub = (T)((double)sum * __longlong_as_double(fix[nb]));
+    if constexpr (WALK && sizeof(T) == 8) {
+        if (fix) dsub.s = (double)sum * __longlong_as_double(fix[nb]);
+    }
+    d = dsub.diagonal(diag);
 }
 
 // FP64 rows take the integer J_b/2 in shared memory, up to this many bonds and
@@ -201,16 +251,18 @@ template <typename T>
 constexpr bool kFixRow = sizeof(T) == 8;
 
 // Bond masks and J_b/2 from the handle's bond table [J (nb) | masks (nb) | sum
-// J / 4 | unit | J/2 in units (nb)]; sm_fix: [nb + 1], or null.
+// J / 4 | unit | J/2 in units (nb) | FP32: sum J / 4 in units 2^32 times as large,
+// their two factors]; sm_fix: [nb + 1], or null.
 template <typename T>
-__device__ __forceinline__ void stage_bonds(const double *__restrict__ bond, int nb, uint64_t *sm_mask, T *sm_half,
+__device__ __forceinline__ void stage_bonds(const double *__restrict__ bond, int nb, uint64_t *sm_mask, BondCoef<T> *sm_coef,
                                             long long *sm_fix = nullptr) {
     const uint64_t *masks = (const uint64_t *)(bond + nb);
     if (sm_fix)
         for (int b = threadIdx.x; b <= nb; b += blockDim.x)
             sm_fix[b] = __double_as_longlong(b < nb ? bond[2 * nb + 2 + b] : bond[2 * nb + 1]);
     for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-        sm_half[b] = (T)(0.5 * bond[b]);
+        sm_coef[b].h = (T)(0.5 * bond[b]);
+        if constexpr (sizeof(T) == 4) sm_coef[b].f = (int)((__double_as_longlong(bond[2 * nb + 2 + b]) + (1ll << 31)) >> 32);
         sm_mask[b] = masks[b];
     }
 }
@@ -218,8 +270,8 @@ __device__ __forceinline__ void stage_bonds(const double *__restrict__ bond, int
 // y = H x on the rows of this CTA (grid-stride tiles of blockDim.x rows);
 // every thread of the CTA calls it (the tile unranking has barriers).
 template <typename T, int NV, bool COHERENT, bool VEC>
-__device__ __forceinline__ void apply_rows(const U1View &u, const uint64_t *sm_mask, const T *sm_half, int nb,
-                                           T jq, const T *x, T *y, uint64_t *sh_range, const long long *fix) {
+__device__ __forceinline__ void apply_rows(const U1View &u, const uint64_t *sm_mask, const BondCoef<T> *sm_coef, int nb,
+                                           const RowDiag<T> &diag, const T *x, T *y, uint64_t *sh_range, const long long *fix) {
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < u.dim; base += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = base + threadIdx.x;
         const RowState rs = unrank_tile(u, base, r, sh_range);
@@ -228,11 +280,10 @@ __device__ __forceinline__ void apply_rows(const U1View &u, const uint64_t *sm_m
         T acc[NV];
 #pragma unroll
         for (int k = 0; k < NV; ++k) acc[k] = T(0);
-        T dsub = T(0);
-        row_flips<T, NV, COHERENT, VEC>(u, s, sm_mask, sm_half, nb, x, acc, dsub, fix);
+        T d;
+        row_flips<T, NV, COHERENT, VEC>(u, s, sm_mask, sm_coef, nb, x, acc, diag, d, fix);
         T xr[NV];
         load_row<T, NV, COHERENT, VEC>(x, r, xr);
-        const T d = jq - dsub;
 #pragma unroll
         for (int k = 0; k < NV; ++k) xr[k] = fma_rn(d, xr[k], acc[k]);
         store_row<T, NV, VEC>(y, r, xr);
