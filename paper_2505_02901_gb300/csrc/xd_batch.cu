@@ -58,11 +58,9 @@ template <typename T, int NV, bool VEC>
 __device__ __forceinline__ void batch_rows_at(const Inst &I, const uint64_t *sm_mask, const BondCoef<T> *sm_coef,
                                            uint64_t *sh_range, int64_t row0, int64_t row1) {
     const U1View &u = I.u;
-    if (threadIdx.x == 0) {
-        uint64_t nh = 1ull << u.P;
-        uint64_t h0 = find_block(u.hi_off, 0, nh - 1, row0);
-        sh_range[0] = h0;
-        sh_range[1] = find_block(u.hi_off, h0, nh - 1, row1 - 1);
+    if (threadIdx.x < 64) {  // as unrank_tile: the first two warps an end each
+        const uint64_t h = u1rows::find_block_warp(u.hi_off, 0, (1ull << u.P) - 1, threadIdx.x < 32 ? row0 : row1 - 1);
+        if ((threadIdx.x & 31) == 0) sh_range[threadIdx.x >> 5] = h;
     }
     __syncthreads();
     const u1rows::RowDiag<T> diag(I.bond, I.nb);

@@ -305,6 +305,19 @@ xd_status sym_correlations(const xd_basis_s *b, const void *psi, xd_dtype dt, co
 xd_status vec_random(int64_t n, uint64_t seed, void *out, xd_dtype dt,
                      cudaStream_t st);
 // block-structured U(1) product (xd_u1_block.cu)
+// Blocks that the block and window kernels are made for.  Smaller ones take the
+// row loop at every width, also from 24 sites on: there the launches, lists and
+// emptier tiles of the others cost more than their work.  One vector of random
+// couplings, us, row loop and the best of the others, FP64 / FP32 / eight FP32:
+// 40-site chain with one spin up (40 rows) 11 and 54 / 15 and 37 / 11 and 33, 8x4
+// J1-J2 with three (4,960) 17 and 62 / 25 and 35 / 17 and 53, 4x6 with six
+// (134,596) 29 and 117 / 28 and 88 / 41 and 132, complete graph of 28 sites with
+// six (376,740) 194 and 670 / 185 and 400 / 231 and 530.  From some 700,000 rows on
+// the dense graphs turn: complete graph of 24 sites with eight (735,471) 307 and
+// 398 / 255 and 192 / 389 and 415; 4x6 with twelve (2,704,156) 458 and 339 / 334 and
+// 167 / 786 and 561.
+constexpr int64_t kRowLoopRows = 1 << 19;
+inline bool large_block(const xd_basis_s *b) { return !b->sym && b->N >= 24 && b->dim_u1 >= kRowLoopRows; }
 bool block_layout_wanted(const xd_basis_s *b);
 xd_status block_layout_build(xd_basis_s *b);
 void block_layout_free(xd_basis_s *b);

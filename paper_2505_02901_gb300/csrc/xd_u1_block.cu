@@ -307,7 +307,7 @@ bool block_layout_wanted(const xd_basis_s *b) {
     // below 24 sites the row loop is faster (us, FP64: 4x5 lattice 33 against 90,
     // 22-site ladder 69 against 164, 23-site chain 77 against 107, 23 sites with
     // 60 random bonds 173 against 316, FP32 115 against 120)
-    if (b->sym || b->N < 24 || b->L < 10) return false;
+    if (!large_block(b) || b->L < 10) return false;
     int ncross = 0;
     for (const Bond &bd : b->bonds) {
         int i = std::min(bd.i, bd.j), j = std::max(bd.i, bd.j);

@@ -414,7 +414,7 @@ int spmm_L(int N) { return std::min(12, N - 12); }
 }  // namespace
 
 bool spmm_layout_wanted(const xd_basis_s *b) {
-    if (b->sym || b->N < 24 || b->nb > 4095) return false;
+    if (!large_block(b) || b->nb > 4095) return false;
     const int L = spmm_L(b->N);
     return L >= 10 && b->N - L <= 26;
 }

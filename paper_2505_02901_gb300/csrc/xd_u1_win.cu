@@ -902,7 +902,7 @@ struct Pack {
     }
 };
 
-bool win_layout_wanted(const xd_basis_s *b) { return !b->sym && b->N >= 24; }
+bool win_layout_wanted(const xd_basis_s *b) { return large_block(b); }
 
 // The passes of the block's graph, the words outside their windows and the
 // tiles; the flip lists follow with the couplings (win_ham_tables).

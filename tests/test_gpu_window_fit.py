@@ -19,8 +19,8 @@ def test_dense_graph_in_a_batch_and_alone(orc):
     """The product in FP64, in FP32 and on eight FP32 vectors, alone and in a batch beside a chain."""
     A = api()
     bonds, J = _dense25()
-    st = orc.enumerate_states(25, 6)
-    ham = A.Hamiltonian(A.Basis(25, 6, bonds), J)
+    st = orc.enumerate_states(25, 8)
+    ham = A.Hamiltonian(A.Basis(25, 8, bonds), J)
     chain = A.Hamiltonian(A.Basis(18, 9, W.chain(18)), np.ones(18))
     st2 = orc.enumerate_states(18, 9)
     rng = np.random.default_rng(3)
