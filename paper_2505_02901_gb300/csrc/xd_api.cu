@@ -494,11 +494,11 @@ static xd_status set_J(xd_ham_s *h, const double *J) {
         memcpy(&buf[2 * b->nb + 2 + k], &f, sizeof f);
     }
     // FP32: sum J/4 in units of 2^(ex - 30), that unit as two factors
-    const long long jq = fits ? llrint(ldexp(0.25 * q, 30 - ex)) : 0;
-    const int half = (ex - 30) / 2;
-    memcpy(&buf[3 * b->nb + 2], &jq, sizeof jq);
-    buf[3 * b->nb + 3] = fits ? ldexp(1.0, half) : 0.0;
-    buf[3 * b->nb + 4] = fits ? ldexp(1.0, ex - 30 - half) : 0.0;
+    const int half = (ex - 30) / 2, jq = fits ? (int)llrint(ldexp(0.25 * q, 30 - ex)) : 0;
+    const float u[2] = {fits ? (float)ldexp(1.0, half) : 0.f, fits ? (float)ldexp(1.0, ex - 30 - half) : 0.f};
+    double *f32 = &buf[(3 * b->nb + 3) / 2 * 2];
+    memcpy(f32, &jq, sizeof jq);
+    memcpy((char *)f32 + 4, u, sizeof u);
     XD_CUDA(cudaMemcpy(h->d_bond, buf.data(), sizeof(double) * buf.size(), cudaMemcpyHostToDevice));
     if (b->blk.ok) XD_TRY(block_ham_tables(h));
     if (b->spmm.ok) XD_TRY(spmm_ham_tables(h));

@@ -235,7 +235,7 @@ struct xd_ham_s {
     xd_basis b = nullptr;
     std::vector<double> J;
     double *d_J = nullptr;          // [nb]
-    double *d_bond = nullptr;       // [J (nb) | bond masks (nb, as uint64) | sum J / 4 | unit | J/2 in units (nb, as int64) | FP32: sum J / 4 (as int64), unit in two factors]
+    double *d_bond = nullptr;       // [J (nb) | bond masks (nb, as uint64) | sum J / 4 | unit | J/2 in units (nb, as int64) | FP32, 16 bytes aligned: sum J / 4 (int32), unit in two factors]
     double *d_part = nullptr;       // reduction partials
     size_t part_bytes = 0;
     double *d_scal = nullptr;       // small device scalars

@@ -146,10 +146,8 @@ struct RowDiag {
 };
 template <>
 struct RowDiag<float> {
-    int jq;
-    float u1, u2;  // the unit in two factors, both normal numbers
-    __device__ __forceinline__ RowDiag(const double *__restrict__ bond, int nb)
-        : jq((int)*(const long long *)(bond + 3 * nb + 2)), u1((float)bond[3 * nb + 3]), u2((float)bond[3 * nb + 4]) {}
+    const int4 *at;  // sum J/4 and the unit in two factors, both normal numbers: read for each row, registers being short
+    __device__ __forceinline__ RowDiag(const double *__restrict__ bond, int nb) : at((const int4 *)(bond + (3 * nb + 3) / 2 * 2)) {}
 };
 template <typename T>
 struct DiagSum {
@@ -161,7 +159,10 @@ template <>
 struct DiagSum<float> {
     int s = 0;
     __device__ __forceinline__ void add(BondCoef<float> c) { s += c.f; }
-    __device__ __forceinline__ float diagonal(const RowDiag<float> &g) const { return (float)(g.jq - s) * g.u1 * g.u2; }
+    __device__ __forceinline__ float diagonal(const RowDiag<float> &g) const {
+        const int4 v = __ldg(g.at);
+        return (float)(v.x - s) * __int_as_float(v.y) * __int_as_float(v.z);
+    }
 };
 
 // The flipping bonds of a row with state s, in ascending order: acc += J_b/2
@@ -251,8 +252,8 @@ template <typename T>
 constexpr bool kFixRow = sizeof(T) == 8;
 
 // Bond masks and J_b/2 from the handle's bond table [J (nb) | masks (nb) | sum
-// J / 4 | unit | J/2 in units (nb) | FP32: sum J / 4 in units 2^32 times as large,
-// their two factors]; sm_fix: [nb + 1], or null.
+// J / 4 | unit | J/2 in units (nb) | at the next multiple of 16 bytes, FP32: sum J / 4
+// in units 2^32 times as large, that unit's two factors]; sm_fix: [nb + 1], or null.
 template <typename T>
 __device__ __forceinline__ void stage_bonds(const double *__restrict__ bond, int nb, uint64_t *sm_mask, BondCoef<T> *sm_coef,
                                             long long *sm_fix = nullptr) {
