@@ -171,7 +171,7 @@ struct WinPassDev {
 
 struct WinLayoutHost {
     bool ok = false;
-    bool spmm32 = false;                     // the FP32 product takes the batched layout (spmm_better)
+    bool spmm32 = false, spmm8 = false;      // the FP32 product (of eight vectors) takes the batched layout (spmm_better)
     std::vector<std::pair<int, int>> pairs;  // distinct bonds
     std::vector<int> pair_of;                // per bond
     std::vector<WinPassDev> pass;
@@ -347,7 +347,7 @@ xd_status passes_tables(xd_ham_s *h);
 xd_status passes_apply_f64(const xd_ham_s *h, const void *x, void *y, cudaStream_t st);
 void pass_layout_free(xd_basis_s *b);
 // FP32 product of sparse graphs on the batched layout (xd_u1_spmm.cu)
-bool spmm_better(const xd_basis_s *b);
+bool spmm_better(const xd_basis_s *b, const std::vector<WinPlan> &plan, bool eight);
 xd_status spmm_apply(const xd_ham_s *h, const void *x, void *y, cudaStream_t st);
 xd_status x64_workspace(xd_ham_s *h, int64_t dim);
 // free the FP64 product's workspace (the next FP64 product allocates it again)

@@ -594,17 +594,62 @@ static xd_status launch_spmm(const xd_ham_s *h, const void *x, void *y, cudaStre
     return XD_OK;
 }
 
-// Sparse graphs, whose products the window passes' fixed cost outweighs: by
-// the estimates of both (this product: 5000 ps a row and 720 a flip, bonds
-// listed twice counted twice).  Measured, this product against the window
-// passes (us): 24-site chain 60 and 100, 26-site chain 194 and 250, 28-site
-// graph of 80 random bonds 2031 and 2450; 28-site chain 699 and 690, 28-site
-// ladder 1596 and 1268, 4x7 lattice 1791 and 1586, 4x8 lattice 31830 and 18130.
-bool spmm_better(const xd_basis_s *b) {
-    if (!b->spmm.ok) return false;
+// Whether the batched layout does the FP32 product faster than the window
+// passes (eight: on eight vectors).  Two estimates; the windows have to win both.
+//
+// The first is for half filling and tens of millions of rows, per row: windows
+// win_cost32, this product 5000 and 720 a flip (eight vectors 28000 and 3600
+// against 26000 a pass and 700 a flip), bonds listed twice counted twice here.
+// us, here and in windows: 28-site chain 699 and 690, ladder 1596 and 1268, 4x7
+// lattice 1791 and 1586, 4x8 lattice 31830 and 18130; eight vectors, 28-site
+// ladder 6545 and 3843, 4x7 8507 and 5649, chain 2572 and 3527.
+//
+// The second adds what counts in blocks of a few million rows and in random
+// graphs: a cost per pass, the padding of its slots and columns, and here the
+// prefix blocks and the bonds' classes.  In us, fitted where the two products
+// are within a factor of 1.7 (114 and 137 of them, 24 to 36 sites): this product
+// to 6%, the windows to 17%.  Measured, us, here and in windows: 4x6 lattice with
+// eight up 107 and 135, 5x5 lattice 286 and 348, 28 sites with 168 random bonds
+// 3040 and 3710, 25 sites with 150 bonds and eight up 207 and 289; eight vectors,
+// 24 sites with 36 random bonds 327 and 374.  Where the batched layout is not built
+// (39 and 40 sites), eight vectors take the row loop: complete graph of 40 sites
+// with seven up 20.9 ms against 25.8 in windows, with eight 93.6 and 92.0, chains
+// half of the windows' time.
+bool spmm_better(const xd_basis_s *b, const std::vector<WinPlan> &plan, bool eight) {
+    const SpmmLayoutHost &s = b->spmm;
+    if (!s.ok) return eight;
+    const int npairs = (int)b->win.pairs.size();
+    const double flips = win_flips(b->N, b->nup, b->nb), pair_flips = win_flips(b->N, b->nup, npairs);
     std::vector<WinPass> passes;
-    for (const WinPassDev &d : b->win.pass) passes.push_back(d.p);
-    return 5000.0 + 720.0 * win_flips(b->N, b->nup, b->nb) <= win_cost32(b->N, b->nup, passes, (int)b->win.pairs.size());
+    for (const WinPlan &d : plan) passes.push_back(d.p);
+    if (eight ? 28000.0 + 3600.0 * flips <= 26000.0 * (double)plan.size() + 700.0 * pair_flips
+              : 5000.0 + 720.0 * flips <= win_cost32(b->N, b->nup, passes, npairs))
+        return true;
+    const double rows = 1e-6 * (double)b->dim_u1, flip = win_flips(b->N, b->nup, 1);
+    double win = 0.0;
+    for (const WinPlan &d : plan) {
+        const int ws = (int)d.p.S.size(), nwb = (int)d.p.bonds.size();
+        double slots = 0.0;  // row slots of the tiles, in millions
+        for (int k = 0; k <= ws; ++k)
+            if (b->nup >= k && b->nup - k <= b->N - ws)
+                slots += 1e-6 * (double)n_choose_k(b->N - ws, b->nup - k) * kWinRows * d.T.k[k].nstep;
+        if (d.p.rows) {
+            win += (d.p.c0 >= 6 ? (eight ? 17.0 : 0.93) : eight ? 29.0 : 8.9) * slots + (eight ? 1.2 : 0.0) * flip * nwb * rows;
+        } else {
+            const double used = win_column_use(b->N, b->nup, (int)d.p.olo.size(), kWinCols[eight ? kWinF32x8 : kWinF32]);
+            win += ((eight ? 29.0 : 5.3) * slots + (eight ? 0.74 : 0.2) * flip * nwb * rows) / used;
+        }
+        win += eight ? 20.0 + 0.47 * nwb : 23.0 + 0.15 * nwb;
+    }
+    double blocks = 0.0;  // prefix blocks, in millions
+    for (int j = std::max(0, b->nup - s.L); j <= std::min(s.P, b->nup); ++j) blocks += 1e-6 * (double)n_choose_k(s.P, j);
+    if (eight)
+        return rows * (flip * (0.9 * s.npost + 1.7 * s.npre + 2.2 * s.ncross) + 3.9 * s.ncsite) +
+                   blocks * (19000.0 + 310.0 * s.npost + 370.0 * s.npre + 350.0 * s.ncross) <=
+               0.97 * win;
+    return 39.0 + rows * (flip * (0.25 * s.npre + 0.53 * s.ncross) + 1.1 * s.ncsite) +
+               blocks * (4900.0 + 170.0 * s.npost + 32.0 * s.npre + 93.0 * s.ncross) <=
+           win;
 }
 
 xd_status spmm_apply(const xd_ham_s *h, const void *x, void *y, cudaStream_t st) {

@@ -931,7 +931,8 @@ xd_status win_layout_build(xd_basis_s *b) {
         }
     }
     XD_TRY(pack.upload(&wl.buf));
-    wl.spmm32 = spmm_better(b);
+    wl.spmm32 = spmm_better(b, plan, false);
+    wl.spmm8 = spmm_better(b, plan, true);
     wl.ok = true;
     return XD_OK;
 }
@@ -1223,17 +1224,10 @@ xd_status win_apply_f32(const xd_ham_s *h, const void *x, void *y, cudaStream_t 
 }
 
 // Eight FP32 vectors: where these passes are estimated faster than the prefix
-// blocks of xd_u1_spmm8.cu (ps a row: 26000 a pass and 700 a flip against
-// 28000 and 3600 a flip, bonds listed twice counted twice).  Measured, here
-// and there (us): 28-site ladder 3843 and 6545, 4x7 lattice 5649 and 8507,
-// 24-site ladder 320 and 375; 28-site chain 3527 and 2572, 24-site chain 276
-// and 154.  Where the tables of a pass do not fit, and where row offsets have 64
-// bits, the prefix blocks stay.
+// blocks of xd_u1_spmm8.cu (spmm_better) and their tables fit (no 64-bit row
+// offsets).
 bool win8_usable(const xd_ham_s *h, const void *x, const void *y) {
-    const xd_basis_s *b = h->b;
-    return h->win_fit[kWinF32x8] && (((uintptr_t)x | (uintptr_t)y) & 15) == 0 &&
-           26000.0 * b->win.pass.size() + 700.0 * win_flips(b->N, b->nup, (int)b->win.pairs.size()) <
-               28000.0 + 3600.0 * win_flips(b->N, b->nup, b->nb);
+    return h->win_fit[kWinF32x8] && !h->b->win.spmm8 && (((uintptr_t)x | (uintptr_t)y) & 15) == 0;
 }
 
 xd_status win8_apply(const xd_ham_s *h, const void *x, void *y, cudaStream_t st) {

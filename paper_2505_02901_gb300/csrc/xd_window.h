@@ -281,7 +281,7 @@ inline std::vector<WinPass> choose_windows(int N, int nup, const std::vector<std
     return out;
 }
 
-// Clocks-free estimate of the FP32 product's time per row in picoseconds:
+// Estimate of the FP32 product's time per row at half filling, in femtoseconds:
 // 4300 a pass (1.4 times that where the lowest sites in the window are few,
 // 1.9 times where the columns are runs of the lowest four sites) and 250 a
 // flip, fitted to chains, ladders and lattices of 24 to 32 sites.
