@@ -601,9 +601,8 @@ void lanczos_forget(xd_ham_s *h, bool all) {
 }
 
 // Launch shape of the cooperative first pass, or false where it does not
-// apply: a U(1) block without the block layouts (its product is the plain
-// row loop), one row per thread with every CTA resident, a device with
-// cooperative launch.
+// apply: a U(1) block that is not large (large_block), one row per thread with
+// every CTA resident, a device with cooperative launch.
 struct LzSmall {
     int grid;
     size_t smem;
@@ -615,7 +614,7 @@ struct LzSmall {
 template <typename T>
 static bool lz_small_shape(const xd_ham_s *h, LzSmall *out) {
     const xd_basis_s *b = h->b;
-    if (b->sym || b->blk.ok || b->spmm.ok || b->dim > (1 << 22)) return false;
+    if (b->sym || large_block(b) || b->dim > (1 << 22)) return false;
     int dev = 0, coop = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) {

@@ -242,7 +242,8 @@ xd_status u1_apply(const xd_ham_s *h, const void *x, void *y, xd_dtype dt, int n
     }
     if (nvec == 8 && dt == XD_F32 && win8_usable(h, x, y)) return win8_apply(h, x, y, st);
     if (nvec == 8 && dt == XD_F32 && spmm8_usable(h, x, y)) return spmm8_apply(h, x, y, st);
-    if (nvec == 1 && h->b->blk.ok) return block_apply(h, x, y, dt, st);
+    // (built below 24 sites for FP32 alone)
+    if (nvec == 1 && h->b->blk.ok && (dt == XD_F32 || h->b->N >= 24)) return block_apply(h, x, y, dt, st);
     if (dt == XD_F64) {
         switch (nvec) {
             case 1: return launch_apply<double, 1>(h, x, y, st);
