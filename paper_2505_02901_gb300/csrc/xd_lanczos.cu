@@ -95,7 +95,8 @@ struct AccOf<float> {
 
 // Flip tables of the cooperative Lanczos passes: 24 bits of row, 8 of bond,
 // after the bond table in shared memory.
-constexpr int kLzTabRow = 24, kLzTabBonds = 256, kLzTabBytes = 128 * 1024;
+constexpr int kLzTabRow = 24, kLzTabBytes = 128 * 1024;
+static_assert(kLzTabBytes / (kThreads * (int)sizeof(uint32_t)) <= 256, "a table's bonds fit in 8 bits");
 template <typename T>
 __host__ __device__ inline size_t lz_tab_at(int nb) {
     return ((size_t)nb * (sizeof(uint64_t) + sizeof(u1rows::BondCoef<T>)) + 15) / 16 * 16;
@@ -293,8 +294,16 @@ __global__ void __launch_bounds__(kThreads) k_lz_axpby2(int64_t n, T *__restrict
 // one vector instead of a chain of table look-ups each.  These passes are
 // bound by the latency of a step: 120 steps of the 16-site ladder 2.27 -> 1.60
 // ms with the table, of the 3x6 lattice (48,620 rows, 72 bonds) 4.05 -> 2.84.
-template <typename T, bool TAB>
+// Without the table (127 bonds and more) FP64 walks the set bits, as the row loop,
+// from 2^17 rows on and takes the bonds in turn below, where the FP64 pipe is not
+// the limit yet.  60 steps of the complete graphs, ms, in turn and walked: 18 sites
+// (48,620 rows) 3.43 and 3.75, 19 sites (92,378) 5.44 and 5.51, 22 sites with seven
+// up (170,544) 12.8 and 5.92, 20 sites (184,756) 12.8 and 5.27.
+enum LzForm { kLzTab, kLzWalk, kLzTurn };
+constexpr int64_t kLzWalkRows = 1 << 17;
+template <typename T, LzForm FORM>
 struct LzRow {
+    static constexpr bool TAB = FORM == kLzTab;
     uint64_t s;
     bool valid;
     int n = 0;
@@ -345,7 +354,7 @@ struct LzRow {
                     if (j + q < n) acc[0] = fma_rn(coef[e[q] >> kLzTabRow].h, x[q], acc[0]);
             }
         } else {
-            u1rows::row_flips<T, 1, true, false>(u1, s, mask, coef, nb, u, acc, diag, dr);
+            u1rows::row_flips<T, 1, true, false, FORM == kLzWalk>(u1, s, mask, coef, nb, u, acc, diag, dr);
         }
         return fma_rn(dr, ur, acc[0]);
     }
@@ -364,7 +373,7 @@ struct LzRow {
 // so all CTAs hold the same alpha, beta and stop decision; CTA 0 records
 // them.  A thread updates only its own row, so only the product's gathers
 // read other CTAs' writes (through L2).
-template <typename T, bool TAB>
+template <typename T, LzForm FORM>
 __global__ void __launch_bounds__(kThreads) k_lz_persist(U1View u1, const double *__restrict__ bond, int nb,
                                                          T *b0, T *b1, T *b2, LzDev *sd, double *pa,
                                                          double *pb, double *pc, double *__restrict__ alpha,
@@ -374,7 +383,7 @@ __global__ void __launch_bounds__(kThreads) k_lz_persist(U1View u1, const double
     __shared__ uint64_t sh_range[2];
     __shared__ double sh_sum[2];
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // this thread's row
-    const LzRow<T, TAB> row(u1, bond, nb, smem, r, sh_range);
+    const LzRow<T, FORM> row(u1, bond, nb, smem, r, sh_range);
     double sig = sd->sig, cz = sd->cz, amax = sd->amax;
     int k = sd->k;
     const int max_iter = sd->max_iter;
@@ -442,7 +451,7 @@ __global__ void __launch_bounds__(kThreads) k_lz_persist(U1View u1, const double
 // barrier a step; the vectors take turns in two buffers.  abc: alpha, beta,
 // coef, [steps] each.  120 steps of the 16-site ladder 3.1 ms as four launches
 // a step, 0.85 ms here; 4x5 lattice (184,756 rows) 12.7 and 8.3 ms.
-template <typename T, bool TAB>
+template <typename T, LzForm FORM>
 __global__ void __launch_bounds__(kThreads) k_lz_persist2(U1View u1, const double *__restrict__ bond, int nb, T *b0, T *b1,
                                                           double sig, int steps, const double *__restrict__ abc,
                                                           T *__restrict__ psi) {
@@ -450,7 +459,7 @@ __global__ void __launch_bounds__(kThreads) k_lz_persist2(U1View u1, const doubl
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint64_t sh_range[2];
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const LzRow<T, TAB> row(u1, bond, nb, smem, r, sh_range);
+    const LzRow<T, FORM> row(u1, bond, nb, smem, r, sh_range);
     T *u = b0, *w = b1;
     T ur = row.valid ? u[r] : T(0), upr = T(0), acc = T(0);
     double cz = 0.0;
@@ -606,10 +615,21 @@ void lanczos_forget(xd_ham_s *h, bool all) {
 struct LzSmall {
     int grid;
     size_t smem;
-    bool tab;  // the rows' flips in shared memory
+    LzForm form;
 };
 
-// Every CTA must be resident: with the flip tables (up to 128 KB a CTA: 127
+// The passes' kernels in a form; FP32 does not walk (kWalkRow).
+template <typename T>
+static const void *lz_kernel(LzForm form, bool second) {
+    constexpr LzForm walk = sizeof(T) == 8 ? kLzWalk : kLzTurn;
+    if (second)
+        return form == kLzTab ? (const void *)k_lz_persist2<T, kLzTab>
+               : form == kLzTurn ? (const void *)k_lz_persist2<T, kLzTurn> : (const void *)k_lz_persist2<T, walk>;
+    return form == kLzTab ? (const void *)k_lz_persist<T, kLzTab>
+           : form == kLzTurn ? (const void *)k_lz_persist<T, kLzTurn> : (const void *)k_lz_persist<T, walk>;
+}
+
+// Every CTA must be resident: with the flip tables (up to 128 KB a CTA: 126
 // bonds) or else without them.
 template <typename T>
 static bool lz_small_shape(const xd_ham_s *h, LzSmall *out) {
@@ -624,15 +644,15 @@ static bool lz_small_shape(const xd_ham_s *h, LzSmall *out) {
     grid_for(1, 1, 1);
     const int64_t need = (b->dim + kThreads - 1) / kThreads;
     for (int tab = 1; tab >= 0; --tab) {
-        if (tab && b->nb > kLzTabBonds) continue;
         const size_t smem = lz_tab_at<T>(b->nb) + (tab ? (size_t)b->nb * kThreads * sizeof(uint32_t) : 0);
-        if (smem > (size_t)(tab ? kLzTabBytes : 48 * 1024)) continue;
-        const void *k1 = tab ? (const void *)k_lz_persist<T, true> : (const void *)k_lz_persist<T, false>;
-        const void *k2 = tab ? (const void *)k_lz_persist2<T, true> : (const void *)k_lz_persist2<T, false>;
+        const int limit = tab ? kLzTabBytes : 48 * 1024;
+        if (smem > (size_t)limit) continue;
+        const LzForm form = tab ? kLzTab : b->dim < kLzWalkRows ? kLzTurn : kLzWalk;
+        const void *k1 = lz_kernel<T>(form, false), *k2 = lz_kernel<T>(form, true);
         int per1 = 0, per2 = 0;
         // the limit, not this block's size: another thread may be about to launch a larger one
-        if (cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, tab ? kLzTabBytes : 48 * 1024) != cudaSuccess ||
-            cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, tab ? kLzTabBytes : 48 * 1024) != cudaSuccess ||
+        if (cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, limit) != cudaSuccess ||
+            cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, limit) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per1, k1, kThreads, smem) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per2, k2, kThreads, smem) != cudaSuccess) {
             cudaGetLastError();
@@ -641,7 +661,7 @@ static bool lz_small_shape(const xd_ham_s *h, LzSmall *out) {
         if (need > (int64_t)std::min(per1, per2) * g_num_sms) continue;
         out->grid = (int)need;
         out->smem = smem;
-        out->tab = tab != 0;
+        out->form = form;
         return true;
     }
     return false;
@@ -658,7 +678,7 @@ static xd_status lanczos_pass1_graph(xd_ham_s *h, int max_iter, uint64_t seed, x
     lw.grid = grid_for(n, kThreads, 8);
     // small blocks whose product is the plain row loop: one cooperative
     // launch for the whole pass (all its CTAs resident at once)
-    LzSmall lzs{0, 0, false};
+    LzSmall lzs{0, 0, kLzTab};
     const bool persist = lz_small_shape<T>(h, &lzs);
     const int pstride = std::max(lw.grid, lzs.grid);  // three arrays of partials
     XD_TRY(ensure_lanczos_partials(h, 3 * pstride));
@@ -720,8 +740,7 @@ static xd_status lanczos_pass1_graph(xd_ham_s *h, int max_iter, uint64_t seed, x
             double *part3 = h->d_lzpart + 2 * pstride;
             void *args[] = {&u1, (void *)&bond, (void *)&nbh, &p0, &p1, &p2, &d_sd, &part1, &part2, &part3, &d_ab,
                             (void *)&d_abb};
-            e = cudaLaunchCooperativeKernel(lzs.tab ? (const void *)k_lz_persist<T, true> : (const void *)k_lz_persist<T, false>,
-                                            dim3(lzs.grid), dim3(kThreads), args, lzs.smem, st);
+            e = cudaLaunchCooperativeKernel(lz_kernel<T>(lzs.form, false), dim3(lzs.grid), dim3(kThreads), args, lzs.smem, st);
             if (e == cudaSuccess) e = cudaMemcpyAsync(h_sd, d_sd, sizeof(LzDev), cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
             if (e != cudaSuccess) {
@@ -851,7 +870,7 @@ static xd_status lanczos_run(xd_ham_s *h, int max_iter, uint64_t seed, xd_dtype 
         }
         double sig = 1.0 / sqrt(nrm2), sig_prev = 0.0, beta_prev = 0.0;
         const int steps = *n_iter;
-        LzSmall lzs{0, 0, false};
+        LzSmall lzs{0, 0, kLzTab};
         if (lz_small_shape<T>(h, &lzs)) {
             // the whole pass in one cooperative launch
             std::vector<double> abc(3 * (size_t)steps);
@@ -868,9 +887,7 @@ static xd_status lanczos_run(xd_ham_s *h, int max_iter, uint64_t seed, xd_dtype 
                 const double *bond = h->d_bond;
                 T *p0 = u, *p1 = w, *out = psi;
                 void *args[] = {&u1, (void *)&bond, &nbh, &p0, &p1, &sig, &n_steps, &d_abc, &out};
-                e = cudaLaunchCooperativeKernel(
-                    lzs.tab ? (const void *)k_lz_persist2<T, true> : (const void *)k_lz_persist2<T, false>, dim3(lzs.grid),
-                    dim3(kThreads), args, lzs.smem, st);
+                e = cudaLaunchCooperativeKernel(lz_kernel<T>(lzs.form, true), dim3(lzs.grid), dim3(kThreads), args, lzs.smem, st);
             }
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
             cudaFree(d_abc);
