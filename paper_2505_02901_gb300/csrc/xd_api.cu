@@ -472,6 +472,7 @@ static xd_status set_J(xd_ham_s *h, const double *J) {
     lanczos_forget(h, false);
     batch_forget(h);  // captured launches hold per-coupling scalars and addresses
     h->J.assign(J, J + b->nb);
+    h->J_fix.assign(b->nb, 0);
     XD_CUDA(cudaMemcpy(h->d_J, J, sizeof(double) * b->nb, cudaMemcpyHostToDevice));
     std::vector<double> buf(3 * b->nb + 5);
     double q = 0.0;
@@ -492,6 +493,7 @@ static xd_status set_J(xd_ham_s *h, const double *J) {
     for (int k = 0; k < b->nb; ++k) {
         const long long f = fits ? llrint(ldexp(0.5 * J[k], 62 - ex)) : 0;
         memcpy(&buf[2 * b->nb + 2 + k], &f, sizeof f);
+        h->J_fix[k] = f;
     }
     // FP32: sum J/4 in units of 2^(ex - 30), that unit as two factors
     const int half = (ex - 30) / 2, jq = fits ? (int)llrint(ldexp(0.25 * q, 30 - ex)) : 0;

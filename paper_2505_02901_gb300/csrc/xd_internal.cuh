@@ -234,6 +234,7 @@ struct xd_basis_s {
 struct xd_ham_s {
     xd_basis b = nullptr;
     std::vector<double> J;
+    std::vector<long long> J_fix;   // J/2 in units of 2^-62 of a power of two above sum |J/2|
     double *d_J = nullptr;          // [nb]
     double *d_bond = nullptr;       // [J (nb) | bond masks (nb, as uint64) | sum J / 4 | unit | J/2 in units (nb, as int64) | FP32, 16 bytes aligned: sum J / 4 (int32), unit in two factors]
     double *d_part = nullptr;       // reduction partials

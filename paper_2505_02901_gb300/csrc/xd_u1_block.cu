@@ -21,7 +21,9 @@
 //       comes from a per-site table indexed by the row's in-class rank.
 // Each thread owns K rows of the block (i = tid + k * 1024) and keeps their
 // accumulators in registers across the three phases.  The diagonal is
-// d_pre(h) + d_post(l) + the cross-bond terms.  Prefix blocks are walked in
+// d_pre(h) + d_post(l) + the cross-bond terms; FP32 sums it in integers, in the
+// units of the row loop (xd_u1_rows.cuh): sums of both signs that cancel to a few
+// J cost 2.8e-7 against 64 bits in FP32 (23 sites, 103 random bonds).  Prefix blocks are walked in
 // ascending order (static round robin), so the blocks reached by flips on
 // low prefix bits are still in L2.
 
@@ -48,6 +50,10 @@ struct BlkParams {
     const uint16_t *ptab;   // [npost_pad][2^L]: rank of l ^ m_b in class, maxblk = no flip
     const uint16_t *xtab;   // [nslot][2^L]: rank of l ^ 2^j_slot in its class
     const double *dpost;    // [2^L]: postfix diagonal, by class-ordered position
+    const int *dpost_fix;   // FP32: twice that, J/2 in integers
+    const long long *fix;   // FP32: J/2 in units 2^-32 times as large, per bond
+    const int4 *unit;       // FP32: (sum J/4, the unit's two factors)
+    int jcross_fix;         // FP32: sum over cross bonds of J/2 in integers
     const int32_t *post;    // [npost] bond ids
     int npost, npost_pad;   // postfix bonds, padded to a multiple of 8 (dummy rows never flip)
     const double *J;        // [nb]
@@ -74,7 +80,7 @@ struct Geo {
 
 template <typename T>
 struct SmemLayout {
-    size_t xs, nbuf, pc, cc, cmeta, pre, site, total;
+    size_t xs, nbuf, pc, cc, cfix, cmeta, pre, site, total;
     __host__ __device__ SmemLayout(const BlkParams &p, int nbufs) {
         size_t o = 0;
         auto al = [&](size_t a) { o = (o + a - 1) / a * a; };
@@ -89,6 +95,9 @@ struct SmemLayout {
         al(16);
         cc = o;
         o += (size_t)p.ncross * sizeof(T);
+        al(16);
+        cfix = o;
+        if (sizeof(T) == 4) o += (size_t)p.ncross * sizeof(int);
         al(16);
         cmeta = o;
         o += (size_t)p.ncross * sizeof(uint32_t);
@@ -120,6 +129,8 @@ __device__ __forceinline__ void stage(T *dst, const T *src, int n) {
     cp_commit();
 }
 
+__host__ __device__ inline int fix32(long long f) { return (int)((f + (1ll << 31)) >> 32); }
+
 template <typename T, int L, int NBUF>
 __global__ void __launch_bounds__(kBT) k_block_apply(BlkParams p, const T *__restrict__ x,
                                                      T *__restrict__ y) {
@@ -132,17 +143,21 @@ __global__ void __launch_bounds__(kBT) k_block_apply(BlkParams p, const T *__res
     T *nbuf = (T *)(smem + lay.nbuf);
     T *pc = (T *)(smem + lay.pc);
     T *cc = (T *)(smem + lay.cc);
+    int *cfix = (int *)(smem + lay.cfix);
     uint32_t *cmeta = (uint32_t *)(smem + lay.cmeta);
+    constexpr bool FIX = sizeof(T) == 4;
     PreEnt<T> *pl = (PreEnt<T> *)(smem + lay.pre);
     int64_t *site = (int64_t *)(smem + lay.site);  // [ncsite][2]: neighbour offset, (n << 1) | req
     __shared__ int sh_npa;
     __shared__ double sh_dpre;
+    __shared__ int sh_dfix;
 
     const U1View &u = p.u;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int k = tid; k < p.npost_pad; k += kBT) pc[k] = k < p.npost ? (T)(0.5 * p.J[p.post[k]]) : T(0);
     for (int q = tid; q < p.ncross; q += kBT) {
         cc[q] = (T)(0.5 * p.J[p.cross[4 * q + 2]]);
+        if (FIX) cfix[q] = fix32(p.fix[p.cross[4 * q + 2]]);
         cmeta[q] = (uint32_t)p.cross[4 * q + 1] | ((uint32_t)p.cross[4 * q + 3] << 8);
     }
 
@@ -159,6 +174,7 @@ __global__ void __launch_bounds__(kBT) k_block_apply(BlkParams p, const T *__res
             // active prefix bonds (ballot compaction) and the prefix diagonal
             int cnt = 0;
             double dpre = 0.0;
+            int dfix = 0;
             for (int base = 0; base < p.npre; base += 32) {
                 const int q = base + lane;
                 bool act = false;
@@ -169,7 +185,12 @@ __global__ void __launch_bounds__(kBT) k_block_apply(BlkParams p, const T *__res
                     b = p.pre[3 * q + 1];
                     Jq = p.J[p.pre[3 * q + 2]];
                     act = ((h >> a) & 1) != ((h >> b) & 1);
-                    dpre += act ? -0.25 * Jq : 0.25 * Jq;
+                    if (FIX) {
+                        const int f = fix32(p.fix[p.pre[3 * q + 2]]);
+                        dfix += act ? -f : f;
+                    } else {
+                        dpre += act ? -0.25 * Jq : 0.25 * Jq;
+                    }
                 }
                 const unsigned bal = __ballot_sync(0xffffffffu, act);
                 if (act) {
@@ -182,10 +203,14 @@ __global__ void __launch_bounds__(kBT) k_block_apply(BlkParams p, const T *__res
                 cnt += __popc(bal);
             }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) dpre += __shfl_xor_sync(0xffffffffu, dpre, o);
+            for (int o = 16; o > 0; o >>= 1) {
+                if (FIX) dfix += __shfl_xor_sync(0xffffffffu, dfix, o);
+                else dpre += __shfl_xor_sync(0xffffffffu, dpre, o);
+            }
             if (lane == 0) {
                 sh_npa = cnt;
-                sh_dpre = dpre + p.jcross;
+                if (FIX) sh_dfix = dfix + p.jcross_fix;
+                else sh_dpre = dpre + p.jcross;
             }
         } else if (warp == 1) {
             for (int c = lane; c < p.ncsite; c += 32) {
@@ -204,8 +229,12 @@ __global__ void __launch_bounds__(kBT) k_block_apply(BlkParams p, const T *__res
         __syncthreads();  // xs complete
 
         T acc[K];
+        int flip[K];  // FP32: sum over the row's cross flips of J/2
 #pragma unroll
-        for (int k = 0; k < K; ++k) acc[k] = T(0);
+        for (int k = 0; k < K; ++k) {
+            acc[k] = T(0);
+            flip[k] = 0;
+        }
         // postfix bonds: target ranks from the bond-major table (compile-time
         // stride; "no flip" points at the zero slot), x from xs, branch free
 #pragma unroll
@@ -243,7 +272,7 @@ __global__ void __launch_bounds__(kBT) k_block_apply(BlkParams p, const T *__res
             }
         }
         // cross bonds: one staged neighbour block per prefix site; a flip adds
-        // J/2 (x_target - x_row), which also takes J/2 off the diagonal
+        // J/2 (x_target - x_row) in FP64, which also takes J/2 off the diagonal
         for (int c = 0; c < p.ncsite; ++c) {
             T *buf = nbuf + (NBUF == 2 ? (c & 1) : 0) * p.maxblk;
             if (NBUF == 2) {
@@ -282,19 +311,27 @@ __global__ void __launch_bounds__(kBT) k_block_apply(BlkParams p, const T *__res
                             if (f) a += cc[q] * (buf[__ldg(p.xtab + (size_t)(meta >> 8) * nlo + (l0 + i))] - xi);
                         } else {
                             const uint32_t r2 = __ldg(p.xtab + (size_t)(meta >> 8) * nlo + (l0 + i));
-                            const T t = cc[q] * (buf[r2] - xi);
+                            const T t = cc[q] * buf[r2];
                             a += f ? t : T(0);
+                            flip[k] += f ? cfix[q] : 0;
                         }
                     }
                     acc[k] += a;
                 }
             }
         }
-        const T dpre = (T)sh_dpre;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const int i = tid + k * kBT;
-            if (i < n) y[off + i] = (dpre + (T)__ldg(p.dpost + l0 + i)) * xs[i] + acc[k];
+            if (i >= n) continue;
+            T d;
+            if constexpr (FIX) {
+                const int4 unit = __ldg(p.unit);
+                d = 0.5f * (float)(sh_dfix + __ldg(p.dpost_fix + l0 + i) - flip[k] - flip[k]) * __int_as_float(unit.y) * __int_as_float(unit.z);
+            } else {
+                d = (T)sh_dpre + (T)__ldg(p.dpost + l0 + i);
+            }
+            y[off + i] = d * xs[i] + acc[k];
         }
     }
 }
@@ -387,8 +424,16 @@ xd_status block_ham_tables(xd_ham_s *h) {
         for (uint32_t l = 0; l < nlo; ++l) by_word[l] += t[((l >> i) ^ (l >> j)) & 1u];
     }
     for (uint32_t g = 0; g < nlo; ++g) dpost[g] = by_word[b->h_lo_list[g]];
-    if (!h->d_dpost) XD_CUDA(dev_malloc((void **)&h->d_dpost, nlo * sizeof(double)));
+    if (!h->d_dpost) XD_CUDA(dev_malloc((void **)&h->d_dpost, nlo * (sizeof(double) + sizeof(int))));
     XD_CUDA(cudaMemcpy(h->d_dpost, dpost.data(), nlo * sizeof(double), cudaMemcpyHostToDevice));
+    if (b->spmm.ok) return XD_OK;  // no FP32 product comes here
+    std::vector<int> fix_by_word(nlo, 0), dfix(nlo);
+    for (int k : b->blk.post) {
+        const int i = b->bonds[k].i, j = b->bonds[k].j, f = fix32(h->J_fix[k]);
+        for (uint32_t l = 0; l < nlo; ++l) fix_by_word[l] += (((l >> i) ^ (l >> j)) & 1u) ? -f : f;
+    }
+    for (uint32_t g = 0; g < nlo; ++g) dfix[g] = fix_by_word[b->h_lo_list[g]];
+    XD_CUDA(cudaMemcpy(h->d_dpost + nlo, dfix.data(), nlo * sizeof(int), cudaMemcpyHostToDevice));
     return XD_OK;
 }
 
@@ -407,10 +452,17 @@ static xd_status launch_block(const xd_ham_s *h, const void *x, void *y, cudaStr
     p.npost_pad = bl.npost_pad;
     p.J = h->d_J;
     p.dpost = h->d_dpost;
+    p.dpost_fix = (const int *)(h->d_dpost + (1u << b->L));
+    p.fix = (const long long *)(h->d_bond + 2 * b->nb + 2);
+    p.unit = (const int4 *)(h->d_bond + (3 * b->nb + 3) / 2 * 2);
     double q = 0.0;
+    p.jcross_fix = 0;
     for (int k = 0; k < b->nb; ++k) {
         int i = std::min(b->bonds[k].i, b->bonds[k].j), j = std::max(b->bonds[k].i, b->bonds[k].j);
-        if (i < b->L && j >= b->L) q += h->J[k];
+        if (i < b->L && j >= b->L) {
+            q += h->J[k];
+            p.jcross_fix += fix32(h->J_fix[k]);
+        }
     }
     p.jcross = 0.25 * q;
     p.pre = bl.d_pre;
