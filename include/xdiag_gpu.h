@@ -283,8 +283,8 @@ xd_status xd_random_vector(int64_t dim, uint64_t seed, void *out,
  * ninst device pointers, each [dim_k][nvec] (16-byte aligned for the
  * eight-vector products), x != y; dtype XD_F32 or XD_F64; nvec in
  * {1, 2, 4, 8}.  With eight FP32 right-hand sides the sparse operators of
- * N >= 24 (up to 96 of them) are done inside the persistent launch by the
- * eight-vector block product.  The tile schedule is chosen by the library's
+ * N >= 24 and 2^19 rows or more (up to 96 of them) are done inside the
+ * persistent launch by the eight-vector block product.  The tile schedule is chosen by the library's
  * autotuner (median of five timings per candidate) on first use of a (set,
  * dtype, nvec, stream) and the launch is replayed from a captured CUDA graph
  * while the pointers are unchanged; new couplings of a member

@@ -16,7 +16,7 @@
 // CUDA graph and replayed while the batch (handles, vectors, dtype, nvec,
 // stream) is unchanged.
 //
-// Eight FP32 right-hand sides, operators of N >= 24: one persistent launch of
+// Eight FP32 right-hand sides, large operators (large_block): one persistent launch of
 // k_batch8 does the small operators and the sparse large ones.  Its work list
 // is every prefix block of the latter (the eight-vector product of
 // xd_u1_spmm8.cu, one block per unit, largest operators first) followed by the

@@ -287,8 +287,10 @@ __global__ void __launch_bounds__(kThreads) k_lz_axpby2(int64_t n, T *__restrict
     }
 }
 
-// The product of one row in the cooperative passes below: the row loop's
-// order and roundings (xd_u1_rows.cuh).  TAB: the row's flips are kept in
+// The product of one row in the cooperative passes below: the row loop's order
+// of flips (xd_u1_rows.cuh); the diagonal in FP64 is a sum of doubles, the row
+// loop's one of integers, so a vector of one pass is the other's bit for bit only
+// because both take LzRow (lz_small_shape).  TAB: the row's flips are kept in
 // shared memory for the whole pass, target row and bond in one word (column
 // tid of [flips][threads]), so that a step's gathers are independent reads of
 // one vector instead of a chain of table look-ups each.  These passes are
@@ -364,10 +366,10 @@ struct LzRow {
 // whose product is the plain row loop, one row per thread: the row's state
 // word is unranked once (LzRow).  A step is two phases separated by grid-wide
 // barriers:
-//   product: w_r = (H u)_r in the row loop's order and roundings, so that the
-//     vectors are those of the second pass bit for bit, with the partial dots
-//     <H u, u> and <up, u>, so that alpha_k = sig <sig H u + cz up, u> (the
-//     modified form) needs no further pass;
+//   product: w_r = (H u)_r by LzRow, as the second pass forms it, so that the
+//     vectors are the same bit for bit, with the partial dots <H u, u> and <up, u>,
+//     so that alpha_k = sig <sig H u + cz up, u> (the modified form) needs no
+//     further pass;
 //   update: w = sig w + cz up - alpha_k sig u, with the partial norms.
 // Every CTA sums the partials itself in the fixed order of warp_sum_parts,
 // so all CTAs hold the same alpha, beta and stop decision; CTA 0 records

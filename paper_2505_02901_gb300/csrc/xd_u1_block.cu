@@ -344,11 +344,12 @@ __global__ void __launch_bounds__(kBT) k_block_apply(BlkParams p, const T *__res
 // 22-site ladder 69 against 164, 23-site chain 77 against 107, 23 sites with 60
 // random bonds 173 against 316), and in FP32 unless the graph is dense and either
 // the prefix blocks are long (here against the row loop, us: 23 sites with 92
-// bonds 147 and 165, complete graphs of 23, 22 and 21 sites 307 and 427, 200 and
-// 215, 96 and 105; 23 sites with 69 bonds 135 and 133, 22 sites with 132 138 and 130,
-// complete graph of 23 sites with eight up, 239 rows to a prefix, 217 and 159) or
-// the block has so few rows that a thread's walk along the bonds is all there is
-// (three up: complete graph of 23 sites 27 and 35, 22 sites with 88 bonds 17 and 17).
+// bonds 162 and 170, complete graphs of 23, 22 and 21 sites 317 and 423, 204 and
+// 213, 95 and 105; before the integer diagonal, which takes a few per cent, 23
+// sites with 69 bonds 135 and 133, 22 sites with 132 138 and 130, complete graph of
+// 23 sites with eight up, 239 rows to a prefix, 217 and 159) or the block has so few
+// rows that a thread's walk along the bonds is all there is (three up: complete
+// graph of 23 sites 27 and 35, 22 sites with 88 bonds 17.6 and 16.9).
 bool block_fp32_below24(const xd_basis_s *b) {
     if (b->sym || b->N < 20 || b->N >= 24) return false;
     const double per = (double)b->dim_u1 / (double)(1ull << b->P);  // rows to a prefix block

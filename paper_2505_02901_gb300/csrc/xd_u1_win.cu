@@ -1,4 +1,4 @@
-// xd_u1_win.cu -- y = H x on large U(1) blocks (N >= 24) in passes over
+// xd_u1_win.cu -- y = H x on large U(1) blocks (large_block) in passes over
 // windows of sites.
 //
 // H = sum of passes, each the bonds inside a window S of at most 12 sites
@@ -31,8 +31,9 @@
 //   32-site chain          31800 -> 18200  34800 -> 20200      10900 ->  9900
 //   28-site ladder          3320 ->  1820   3890 ->  2090       1600 ->  1270
 //   24-site lattice 4x6      256 ->   199    294 ->   282        146 ->   138
-// At the 4x8 lattice a pass moves 14.4 GB (2.2 ms at the measured copy rate)
-// and takes 6 to 8 ms with the load/store unit 70% busy.
+// At the 4x8 lattice a pass moves 14.4 GB if every value crosses once (2.2 ms at
+// the measured copy rate), 17.9 on average by the counters of the 4x7 lattice, and
+// takes 5.5 to 9 ms with the load/store unit 58 to 65% busy.
 //
 // Arithmetic: FP64 input and output (the paper's precision) without FP64
 // arithmetic per element (GB300's FP64 pipe is a small fraction of its FP32
@@ -546,18 +547,29 @@ __device__ __forceinline__ void tile_in(const WinParams &p, const WinTile &T, co
     }
 }
 
-// One pass, one CTA per SM.  It walks the tiles blockIdx.x, blockIdx.x +
-// gridDim.x, ... (ascending k, so the lists are loaded once per k).  Two warps
-// look up the row offsets of the tiles and copy them into two buffers in turn,
-// one tile ahead; thirty warps flip, a step being sixteen rows, two to each four lanes.
+// One pass, one CTA per SM.  It walks the tiles of its runs (win_divide; popcount
+// by popcount, so the lists are loaded once per run) in three roles: one warp plans
+// (win_next: the shape of tile i + 2), six look up row offsets (tile i + 1) and copy
+// (tile i), seventeen flip, a step being sixteen rows, two to each four lanes.
+//
+// What may be written again, and what allows it: a tile's buffer (two, by i & 1)
+// once the flipping warps have arrived at kBarEmpty of tile i - 2, for which the
+// copying warps wait before tile i; the ring's shapes (four, by i & 3), written by
+// the planning warp for tile i + 2 after kBarCopy of tile i, which the copying warps
+// reach only then, so that tile i - 2 is done with; row offsets and ncols (three or
+// two sets, and four, by the number of their last change, gen), written for tile
+// i + 1 while tiles i and i - 1 are read, or with two sets for tile i before it is
+// copied.  The flipping warps take tile i after kBarFull, for which the copying
+// warps arrive when their copies are there; the lists and the rows kind's sums in
+// the tile's place go between two kBarFlip of the flipping warps alone.  All roles
+// walk the same tiles, so every wait has its arrivals.
+//
 // Columns kind: a step reads the row's earlier sums (acc, y's own memory)
 // before its flips and writes the new ones after them, 32 bytes per row and
 // access.  Rows kind: memory runs along the rows, whose order the steps do not
 // follow, so the sums stay in registers until no row reads the tile any more,
-// go into the tile's place and out from there.  The two roles meet in hardware
-// barriers, each tile's buffer with one for "copied" and one for "done with";
-// both roles walk the same tiles, so every wait has its arrivals.  I: uint32
-// row offsets below 2^32 rows.
+// go into the tile's place and out from there.  I: uint32 row offsets below 2^32
+// rows.
 template <class Pol, bool ROWS, bool BOND, int NVS, typename I>
 __device__ __forceinline__ void win_pass(const WinParams &p, const typename Pol::V *__restrict__ x,
                                          typename Pol::Acc *acc, typename Pol::Y *y) {
@@ -910,17 +922,18 @@ xd_status win_layout_build(xd_basis_s *b) {
     WinLayoutHost &wl = b->win;
     grid_for(1, 1, 1);
     wl.pairs = win_pairs((const int32_t *)b->bonds.data(), b->nb, &wl.pair_of);
-    const std::vector<WinPlan> plan = win_plan(b->N, b->nup, wl.pairs, g_num_sms);
+    std::vector<WinPlan> plan = win_plan(b->N, b->nup, wl.pairs, g_num_sms);
     wl.pass.resize(plan.size());
     Pack pack;
     for (size_t ip = 0; ip < plan.size(); ++ip) {
-        const WinPlan &s = plan[ip];
+        WinPlan &s = plan[ip];
         WinPassDev &d = wl.pass[ip];
         d.p = s.p;
         pack.add(&d.d_ohi, s.T.ohi);
         pack.add(&d.d_olo, s.T.olo);
         pack.add(&d.d_olo_off, s.T.olo_off);
         pack.add(&d.d_whi, s.T.whi);
+        s.T.ohi = s.T.olo = std::vector<uint64_t>();  // up to a hundred MB at 40 sites
         for (int q = 0; q < kWinForms; ++q) {
             d.nseg[q] = (int)s.segs[q].size();
             d.nctas[q] = (int)s.ctas[q].size() - 1;
