@@ -54,7 +54,7 @@ using u1rows::BondCoef;
 using u1rows::find_block;
 
 // Rows [row0, row1) of instance I (bond table staged in sm_mask / sm_coef).
-template <typename T, int NV, bool VEC>
+template <typename T, int NV, bool WALK, bool VEC>
 __device__ __forceinline__ void batch_rows_at(const Inst &I, const uint64_t *sm_mask, const BondCoef<T> *sm_coef,
                                            uint64_t *sh_range, int64_t row0, int64_t row1) {
     const U1View &u = I.u;
@@ -75,8 +75,7 @@ __device__ __forceinline__ void batch_rows_at(const Inst &I, const uint64_t *sm_
 #pragma unroll
         for (int q = 0; q < NV; ++q) acc[q] = T(0);
         T d;
-        // in turn: walked bits spill in k_batch8, whose registers the prefix blocks take
-        u1rows::row_flips<T, NV, false, VEC, false>(u, s, sm_mask, sm_coef, I.nb, x, acc, diag, d);
+        u1rows::row_flips<T, NV, false, VEC, WALK>(u, s, sm_mask, sm_coef, I.nb, x, acc, diag, d);
         T xr[NV];
         u1rows::load_row<T, NV, false, VEC>(x, r, xr);
 #pragma unroll
@@ -85,14 +84,18 @@ __device__ __forceinline__ void batch_rows_at(const Inst &I, const uint64_t *sm_
     }
 }
 
-// in 16-byte pieces where the instance's vectors allow it
-template <typename T, int NV>
+// in 16-byte pieces where the instance's vectors allow it.  The bonds in turn
+// (k_batch8, whose registers the prefix blocks take, spills where it walks their
+// set bits, and full batches are slower: 23 sites with 100 bonds 388 us in turn, 514
+// in the row loop, which walks), except (WALK) eight FP32 columns of a few rows in
+// all, where a thread's chain of look-ups is what takes the time.
+template <typename T, int NV, bool WALK>
 __device__ __forceinline__ void batch_rows(const Inst &I, const uint64_t *sm_mask, const BondCoef<T> *sm_coef,
                                            uint64_t *sh_range, int64_t row0, int64_t row1) {
     if (u1rows::kVecRow<T, NV> && (((uintptr_t)I.x | (uintptr_t)I.y) & 15) == 0)
-        batch_rows_at<T, NV, u1rows::kVecRow<T, NV>>(I, sm_mask, sm_coef, sh_range, row0, row1);
+        batch_rows_at<T, NV, WALK, u1rows::kVecRow<T, NV>>(I, sm_mask, sm_coef, sh_range, row0, row1);
     else
-        batch_rows_at<T, NV, false>(I, sm_mask, sm_coef, sh_range, row0, row1);
+        batch_rows_at<T, NV, WALK, false>(I, sm_mask, sm_coef, sh_range, row0, row1);
 }
 
 // Instance of global tile t: the last with tile0 <= t.
@@ -105,8 +108,8 @@ __device__ __forceinline__ int batch_find(const Inst *__restrict__ inst, int nin
     return lo;
 }
 
-template <typename T, int NV>
-__global__ void k_batch(const Inst *__restrict__ inst, int ninst, int64_t ntiles, int tile_rows) {
+template <typename T, int NV, bool WALK>
+__device__ __forceinline__ void batch_tiles(const Inst *__restrict__ inst, int ninst, int64_t ntiles, int tile_rows) {
     __shared__ uint64_t sm_mask[kMaxBatchBonds];
     __shared__ BondCoef<T> sm_coef[kMaxBatchBonds];
     __shared__ int sh_k;
@@ -122,9 +125,22 @@ __global__ void k_batch(const Inst *__restrict__ inst, int ninst, int64_t ntiles
             cur = k;
         }
         const int64_t row0 = (t - I.tile0) * tile_rows;
-        batch_rows<T, NV>(I, sm_mask, sm_coef, sh_range, row0, min(row0 + (int64_t)tile_rows, I.u.dim));
+        batch_rows<T, NV, WALK>(I, sm_mask, sm_coef, sh_range, row0, min(row0 + (int64_t)tile_rows, I.u.dim));
         __syncthreads();
     }
+}
+
+template <typename T, int NV, bool WALK>
+__global__ void k_batch(const Inst *__restrict__ inst, int ninst, int64_t ntiles, int tile_rows) {
+    batch_tiles<T, NV, WALK>(inst, ninst, ntiles, tile_rows);
+}
+
+// Eight FP32 columns in turn: 40 registers, three CTAs of 512 threads to an SM (eight
+// blocks of 26,334 rows, 66 bonds: 47.5 us, 57.5 in 43 registers).
+template <>
+__global__ void __launch_bounds__(512, 3) k_batch<float, 8, false>(const Inst *__restrict__ inst, int ninst, int64_t ntiles,
+                                                                   int tile_rows) {
+    batch_tiles<float, 8, false>(inst, ninst, ntiles, tile_rows);
 }
 
 // One large operator of the fused launch.
@@ -203,7 +219,7 @@ __global__ void __launch_bounds__(sp8::kT8, 2) k_batch8(const __grid_constant__ 
                 cur_small = k;
             }
             const int64_t row0 = (tt - I.tile0) * a.tile_rows;
-            batch_rows<float, 8>(I, sm_mask, sm_coef, sh_range, row0, min(row0 + (int64_t)a.tile_rows, I.u.dim));
+            batch_rows<float, 8, false>(I, sm_mask, sm_coef, sh_range, row0, min(row0 + (int64_t)a.tile_rows, I.u.dim));
         }
         __syncthreads();  // unit done: shared state may be overwritten
     }
@@ -217,6 +233,11 @@ __global__ void __launch_bounds__(sp8::kT8, 2) k_batch8(const __grid_constant__ 
     }
 }
 
+// Eight FP32 columns walk below this many rows in all row tiles (us, walked and in
+// turn: 36-site chain with one up 10 and 19, 16-site ladder 10.6 and 14.6, eight
+// blocks of 2,024 rows and 276 bonds 33 and 337 in prefix blocks).
+constexpr int64_t kBatchWalkRows = 1 << 15;
+
 struct Plan {
     std::vector<const xd_ham_s *> hs;
     std::vector<const void *> xs;
@@ -227,7 +248,7 @@ struct Plan {
     int nvec;
     cudaStream_t st;
     Inst *d_inst = nullptr;
-    int64_t ntiles = 0;
+    int64_t ntiles = 0, rest_rows = 0;
     int threads = 256, tile_rows = 1024, grid = 1;
     // fused launch (big non-empty)
     std::vector<Big8> hbig;
@@ -249,9 +270,9 @@ void free_plan(Plan *p) {
 std::mutex g_mu;
 std::vector<Plan *> g_plans;
 
-template <typename T, int NV>
+template <typename T, int NV, bool WALK = false>
 void launch(const Plan &p, cudaStream_t st) {
-    k_batch<T, NV><<<p.grid, p.threads, 0, st>>>(p.d_inst, (int)p.rest.size(), p.ntiles, p.tile_rows);
+    k_batch<T, NV, WALK><<<p.grid, p.threads, 0, st>>>(p.d_inst, (int)p.rest.size(), p.ntiles, p.tile_rows);
 }
 
 // the row tiles and prefix blocks
@@ -279,7 +300,9 @@ xd_status launch_fused(const Plan &p, cudaStream_t st) {
             case 1: launch<float, 1>(p, st); break;
             case 2: launch<float, 2>(p, st); break;
             case 4: launch<float, 4>(p, st); break;
-            default: launch<float, 8>(p, st);
+            default:
+                if (p.rest_rows < kBatchWalkRows) launch<float, 8, true>(p, st);
+                else launch<float, 8>(p, st);
         }
     }
     XD_CUDA(cudaGetLastError());
@@ -296,6 +319,7 @@ xd_status launch_any(const Plan &p, cudaStream_t st) {
 xd_status build_table(Plan *p) {
     std::vector<Inst> h(p->rest.size());
     int64_t tiles = 0;
+    p->rest_rows = 0;
     for (size_t q = 0; q < p->rest.size(); ++q) {
         const int k = p->rest[q];
         const xd_ham_s *hm = p->hs[k];
@@ -306,6 +330,7 @@ xd_status build_table(Plan *p) {
         h[q].y = p->ys[k];
         h[q].tile0 = tiles;
         tiles += (hm->b->dim + p->tile_rows - 1) / p->tile_rows;
+        p->rest_rows += hm->b->dim;
     }
     p->ntiles = tiles;
     const int64_t units = p->ubig + tiles;
